@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "cut.cuh"
 #include "gen.cuh"
 #include "sweep.cuh"
 #include "td_internal.h"
@@ -54,7 +55,7 @@ struct td_network {
   int32_t nslots = 0;
   td::FinalArgs fin{};
   int64_t fscr_elems = 0;       // final-contraction scratch per shot (largest candidate layout)
-  int smem_optin = 0;
+  int smem_optin = 0, smem_sm = 0;
   int32_t chunk_rows = td::kChunkRows;   // rows per Gram / update job
   size_t bytes = 0;
   int64_t launches_per_wave = 0;
@@ -187,8 +188,7 @@ static void final_layout(td_network* net, int threads, bool allow_smem = true) {
       mV = std::max<int64_t>(mV, (int64_t)m * td::bank_ld32(m, g));
     }
   }
-  // QR-reduced cuts (n >= m): the copy of M^T (n x m, ld n), the m x m factor R and V with the
-  // leading dimensions of an m x m Jacobi, and the FP32-preconditioning scratch
+  // columns of a cut's factor (cut_ldl)
   int64_t mR = 0;
   {
     const int m_max = cm * Dm;
@@ -199,8 +199,7 @@ static void final_layout(td_network* net, int threads, bool allow_smem = true) {
   }
   int64_t mQ = (int64_t)cmx * Dm * 2 * cm * Dm;
   {
-    // wide cuts (n < m): M (m x n) with the leading dimension of an n-column Jacobi (in the
-    // QR copy's region) and its n x n rotation (in V's region)
+    // copies of a cut (n < m)
     const int m_max = cm * Dm;
     for (int m = 2; m <= m_max; ++m)
       for (int n = 1; n < m; ++n) {
@@ -218,20 +217,25 @@ static void final_layout(td_network* net, int threads, bool allow_smem = true) {
   auto wtake = [&](int64_t n) { int64_t r = wacc; wacc += (n + 3) / 4 * 4; return r; };
   net->fin.w_F = wtake(mF);
   net->fin.w_W = wtake(mW);
+  net->fin.W_elems = mW;
   net->fin.w_MT = wtake(mMT);
   net->fin.w_C0 = wtake(mC);
   net->fin.w_C1 = wtake(mC);
   net->fin.w_s = wtake(mS);
   net->fin.w_ord = wtake(mOrd);
-  // the QR copy is dead once R is extracted, before the preconditioning scratch is used
   net->fin.w_Q = wtake(std::max<int64_t>(mQ, (mP + 3) / 4 * 4 + mT));
-  net->fin.w_P = net->fin.w_Q;
-  net->fin.w_T = net->fin.w_Q + (mP + 3) / 4 * 4;
   net->fin.w_R = wtake(mR);
   net->fin.work_elems = wacc;
-  net->fin.precond = (P.precision == TD_FP64) ? 0 : 1;
-  const size_t static_smem = 8 * 1024;   // k_final's own shared arrays
-  net->fin.use_smem = (allow_smem && (size_t)wacc * net->felem + static_smem <= (size_t)net->smem_optin) ? 1 : 0;
+  net->fin.use_smem = (allow_smem && (size_t)wacc * net->felem + td::kFinalStaticSmem <= (size_t)net->smem_optin) ? 1 : 0;
+  {
+    // the largest cut that truncates: small arrays, vectors and FP32 columns
+    const int m_max = cm * Dm, n_max = (int)(cmx * Dm * 2);
+    const int64_t need = td::CutBuf::small_bytes(m_max, n_max, cm) + td::CutBuf::vec_bytes(m_max, n_max, cm, true) +
+                         4 * (int64_t)td::cut_ldl(threads, m_max) * m_max;
+    net->fin.cut_need = (int32_t)std::min<int64_t>(need, 1 << 30);
+    net->fin.smem_sm = net->smem_sm;
+    net->fin.smem_block = net->smem_optin;
+  }
   int64_t acc = 0;
   auto take = [&](int64_t n) { int64_t r = acc; acc += (n + 3) / 4 * 4; return r; };
   net->fin.off_mps0 = take(mps_stride * P.nx);
@@ -315,16 +319,17 @@ static td_status finish_build(td_network* net, const td_options& o, td_network**
   // final-contraction scratch per shot (elements of the accumulation type): the boundary
   // MPS (two buffers) in global memory, and the work region of one block -- in shared
   // memory when it fits, otherwise after the MPS in global memory.  Block size of k_final:
-  // 512 threads once the widest cut has >= 128 columns (more lanes per column pair in the
-  // Jacobi steps: rotated d=9, chi=16, chi_mps=8 runs 1.9x faster), 256 below (no gain at 64
-  // columns); td_network_tune may pick another of kFinalThreads.  The scratch is sized for
+  // 512 threads (128 registers) once the widest cut has >= 128 columns, whose FP32 copy the pivoted QR
+  // of a cut then keeps in registers (cut.cuh); 256 below, where 64 x 128 fits 256 threads
+  // and three blocks an SM overlap; td_network_tune may pick another of kFinalThreads.  The scratch is sized for
   // the largest layout of all candidates.
   int dev = 0;
   net->smem_optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&net->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+      cudaDeviceGetAttribute(&net->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&net->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) {
     cudaGetLastError();
-    net->smem_optin = 0;
+    net->smem_optin = net->smem_sm = 0;
   }
   int64_t acc = 0;
   for (int th : kFinalThreads)
@@ -911,7 +916,6 @@ static td_status prepare_reverse(td_network* net, int64_t B) {
   td::FinalArgs& G = net->gfin;
   G = net->fin;
   G.use_smem = 0;
-  G.precond = 0;
   G.off_work = (net->fin.off_mps1 + mA * P.nx + 3) / 4 * 4;
   G.scratch_elems = G.off_work + net->fin.work_elems;
   G.rec_stride = fin_stride; G.rec_slot = fin_slot;

@@ -1,0 +1,869 @@
+// Truncation of one zip-up cut of the final contraction: the kept left singular vectors U of
+// M (m x n) and the carry U^T M, from A = M^T (n x m, column-major, FP64), by one block.
+//
+// What bounds it: GB300 issues ~2 FP64 FMAs per clock and SM but 128 in FP32, so a cut costs what
+// its FP64 operations cost.  A one-sided Jacobi SVD of the whole matrix spends ~90 m^3 of them
+// where a cut keeps k << m vectors and, inside the kept space, any orthonormal basis will do (a
+// rotation of it is a gauge of the boundary MPS).  Three paths, in the order in which they are tried:
+//   * cut_topk (min(m, n) > chi_mps): FP32 finds where the leading space is, FP64 puts it right.
+//       1. FP32 Householder QR with column pivoting of A (Golub & Van Loan, Matrix Computations,
+//          4th ed., Alg. 5.4.1), stopped where the pivot falls below 1e-3 of the k-th: r <= min(m, n)
+//          rows of R (typically 0.6 m).
+//       2. FP32 one-sided Jacobi on the r columns of R^T: no rotations of V to accumulate (the
+//          rotated, normalised columns are the right singular vectors of R) and, on the graded
+//          factor of the pivoted QR, 4-6 sweeps instead of 12-22 (Drmac and Veselic, "New fast
+//          and accurate Jacobi SVD algorithm I", 2008).
+//       3. Newton's method on the invariant subspace in FP64: with V the k leading vectors,
+//          P = A V, C = A^T P, E = C - V (V^T C) (all FP64), the first-order correction off the
+//          space is, in the FP32 singular basis,
+//          T = e + sum_i v_i (v_i . e) rho_i / (1 - rho_i), e = E / theta_j, rho_i = sigma_i^2 / theta_j
+//          (FP32: T needs no more digits than it corrects).  Each pass gains the 5-7 digits of the
+//          FP32 basis, so two passes reach FP64 accuracy; V is re-orthonormalised by one
+//          Newton-Schulz step per pass.  FP64 work 10 n m k.
+//     It applies where FP32 resolves the cut: sigma_k - sigma_{k+1} clearly above the multiplet
+//     rule's threshold and sigma_k >= 1e-5 sigma_1; and it checks itself (the residual has to
+//     fall to FP64 rounding).
+//   * cut_rank (rank <= chi_mps: nothing to truncate): FP64 pivoted QR of M, stopped at the first
+//     pivot below svd_cutoff times the largest: U = Q, carry = R.  No SVD.
+//   * cut_full (steep spectra, cuts inside a multiplet): as 1 and 2 in FP64 throughout; every
+//     singular value, so the keep rule is decided on them.
+// Measured against numpy's SVD on 130 cuts of the tests' networks: U U^T M of cut_topk differs by
+// <= 6e-14 sigma_1 (median 2e-15).
+//
+// Data that one step writes and the next reads (norms, pivots, columns, vectors) is kept in
+// registers or shared memory: L1 does not hold written lines, so through global memory each such
+// exchange is an L2 round trip, and these loops are chains of them.
+#pragma once
+
+#include "team.cuh"
+
+namespace td {
+
+// FP32 value of x 2^-E, truncated to 24 bits, from the bit pattern (integer pipes only; below the
+// FP32 normal range: 0).
+__device__ __forceinline__ float cut_f32(double x, int E) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7FFu) - 1023 - E + 127;
+  if (e <= 0) return 0.0f;
+  return __uint_as_float((hi & 0x80000000u) | ((unsigned)e << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+}
+
+// Largest biased exponent of the n x m column-major matrix A, through a shared int.
+__device__ __forceinline__ int cut_max_exponent(const Team& tm, const double* A, int lda, int n, int m, int* slot) {
+  if (tm.tid == 0) *slot = 0;
+  tm.sync();
+  unsigned mx = 0u;
+  const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
+  for (int c = warp; c < m; c += nw)
+    for (int i = lane; i < n; i += 32) mx = max(mx, (unsigned)__double2hiint(A[(size_t)c * lda + i]) & 0x7FFFFFFFu);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0) atomicMax(slot, (int)mx);
+  tm.sync();
+  const int e = *slot >> 20;
+  tm.sync();
+  return e;
+}
+
+// Sums of N (a power of two <= 32) values over the warp: lane l ends with the sum of value
+// l / (32 / N) (each exchange halves the values a lane carries: N shuffles instead of 5 N).
+template <int N, typename R>
+__device__ __forceinline__ R cut_warp_sums(R (&v)[N], int lane) {
+#pragma unroll
+  for (int half = N / 2, off = 16; half >= 1; half >>= 1, off >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const R send = up ? v[i] : v[i + half];
+      const R keep = up ? v[i + half] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+#pragma unroll
+  for (int off = 16 / N; off >= 1; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+  return v[0];
+}
+
+// Pivot keys: norm^2 (the FP32 value, or the upper word of the FP64 one: non-negative, so ordered as
+// integers) with its lowest bits replaced by the column, lower columns first; 0: no column left.
+// The keys only choose the pivot.
+constexpr unsigned kCutColMask = 0x7FFu;   // up to 2048 columns
+__device__ __forceinline__ unsigned cut_key(float norm2, int c) {
+  return (__float_as_uint(fmaxf(norm2, 0.f)) & ~kCutColMask) | (kCutColMask - (unsigned)c);
+}
+__device__ __forceinline__ unsigned cut_key(double norm2, int c) {
+  return ((unsigned)__double2hiint(norm2 > 0.0 ? norm2 : 0.0) & ~kCutColMask) | (kCutColMask - (unsigned)c);
+}
+__device__ __forceinline__ unsigned cut_best_key(const unsigned* keys, int nw, int lane) {
+  return __reduce_max_sync(0xffffffffu, lane < nw ? keys[lane] : 0u);
+}
+
+// Householder QR with column pivoting of the FP32 copy of A (n x m FP64, scaled by 2^-expo), the
+// copy in registers: warp w holds columns w, w + nw, ... (CPW of them), a lane rows lane + 32 t
+// (t < RPL).  Two barriers per step: the pivot is known after the first, its column (written by its
+// warp) after the second; dot products and norms of a warp's columns are reduced together.  The norm
+// of a column after step j is its norm before it, summed afresh, minus R[j][c]^2.  Stops at the
+// first pivot norm^2 <= max(rel2 * (that of the k-th pivot), abs2 * (that of the first)) or after
+// `most` steps; L[j * ldl + c] = R[j][c].  vcol: n rounded up to 32, + 2 floats; keys: nw.
+// Measured (64 x 128, 256 threads): see DESIGN; the version with the copy in memory took 10x.
+template <int CPW, int RPL>
+__device__ __noinline__ int cut_qrcp_reg(Team tm, const double* A, int lda, int n, int m, int k, int expo, float rel2,
+                                         float abs2, int most, float* L, int ldl, float* vcol, unsigned* keys) {
+  const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
+  float a[CPW][RPL];
+  unsigned taken = 0u;
+#pragma unroll
+  for (int u = 0; u < CPW; ++u) {
+    const int c = warp + u * nw;
+    if (c >= m) taken |= 1u << u;
+#pragma unroll
+    for (int t = 0; t < RPL; ++t) {
+      const int i = lane + 32 * t;
+      a[u][t] = (c < m && i < n) ? cut_f32(A[(size_t)c * lda + i], expo) : 0.f;
+    }
+  }
+  {
+    unsigned key = 0u;
+#pragma unroll
+    for (int u = 0; u < CPW; ++u) {
+      float s = 0.f;
+#pragma unroll
+      for (int t = 0; t < RPL; ++t) s += a[u][t] * a[u][t];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (!((taken >> u) & 1u)) key = max(key, cut_key(s, warp + u * nw));
+    }
+    if (lane == 0) keys[warp] = key;
+  }
+  const int q = n < m ? n : m, nv = (n + 31) & ~31;
+  float d02 = 0.f, dk2 = 0.f;
+  int j = 0;
+  for (; j < q && j < most; ++j) {
+    tm.sync();
+    const unsigned key = cut_best_key(keys, nw, lane);
+    const int p = (int)(kCutColMask - (key & kCutColMask));
+    const float g2 = __uint_as_float(key & ~kCutColMask);
+    if (j == 0) d02 = g2;
+    if (j < k) dk2 = g2;
+    if (key == 0u || !(g2 > 0.f) || g2 <= rel2 * dk2 || g2 <= abs2 * d02) break;
+    if (warp == p % nw) {   // the pivot column becomes the reflector
+      const int pu = p / nw;
+      float x[RPL], s = 0.f, x0 = 0.f;
+#pragma unroll
+      for (int t = 0; t < RPL; ++t) {
+        x[t] = 0.f;
+#pragma unroll
+        for (int u = 0; u < CPW; ++u) x[t] = u == pu ? a[u][t] : x[t];
+        const int i = lane + 32 * t;
+        if (i < j) x[t] = 0.f;
+        s += x[t] * x[t];
+        if (i == j) x0 = x[t];
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      x0 = __shfl_sync(0xffffffffu, x0, j & 31);
+      const float nrm = sqrtf(s), alpha = x0 >= 0.f ? -nrm : nrm;
+#pragma unroll
+      for (int t = 0; t < RPL; ++t) {
+        const int i = lane + 32 * t;
+        if (i < nv) vcol[i] = i == j ? x0 - alpha : x[t];
+      }
+      if (lane == 0) {
+        vcol[nv] = s > 0.f ? 1.f / (s + fabsf(x0) * nrm) : 0.f;   // 2 / v.v
+        vcol[nv + 1] = alpha;
+      }
+    }
+    tm.sync();
+    float v[RPL];
+#pragma unroll
+    for (int t = 0; t < RPL; ++t) v[t] = lane + 32 * t < nv ? vcol[lane + 32 * t] : 0.f;
+    const float tau = vcol[nv], alpha = vcol[nv + 1];
+    float sums[2 * CPW];
+#pragma unroll
+    for (int u = 0; u < CPW; ++u) {
+      sums[u] = 0.f;
+      sums[CPW + u] = 0.f;
+#pragma unroll
+      for (int t = 0; t < RPL; ++t) {
+        sums[u] += v[t] * a[u][t];
+        const float x = lane + 32 * t < j ? 0.f : a[u][t];
+        sums[CPW + u] += x * x;
+      }
+    }
+    const float mine = cut_warp_sums<2 * CPW, float>(sums, lane);
+    constexpr int STEP = 32 / (2 * CPW);
+    unsigned best = 0u;
+#pragma unroll
+    for (int u = 0; u < CPW; ++u) {
+      const int c = warp + u * nw;
+      const float w = tau * __shfl_sync(0xffffffffu, mine, u * STEP);
+      const float s = __shfl_sync(0xffffffffu, mine, (CPW + u) * STEP);
+      float top = 0.f;
+#pragma unroll
+      for (int t = 0; t < RPL; ++t) {
+        a[u][t] -= w * v[t];
+        if (lane + 32 * t == j) top = a[u][t];
+      }
+      const bool on = !((taken >> u) & 1u) && c != p;
+      if (lane == (j & 31)) {
+        if (c < m) L[(size_t)j * ldl + c] = on ? top : (c == p ? alpha : 0.f);
+        if (on) best = max(best, cut_key(s - top * top, c));
+      }
+      if (c == p) taken |= 1u << u;
+    }
+    if (lane == (j & 31)) keys[warp] = best;
+  }
+  tm.sync();
+  return j;
+}
+
+// The same factorisation of A (n x m, lda; destroyed) in memory, FP32 or FP64: four columns at a time,
+// one barrier per step (every warp forms the reflector from the pivot column, which is only read).
+// vr != null: vr[4 j ..] = (v_0, 2 / v.v, R[j][piv_j], piv_j) of reflector j, whose tail stays in
+// column piv_j of A.  left: the largest remaining norm^2 over the first.  nr: 2 m values, keys: 2 nw.
+template <typename R>
+__device__ __noinline__ int cut_qrcp(Team tm, R* A, int lda, int n, int m, int k, R rel2, R abs2, int most, R* L, int ldl,
+                                     R* vr, unsigned char* taken, unsigned* keys, R& left) {
+  constexpr int CB = 4;
+  const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
+  {
+    unsigned key = 0u;
+    for (int c = warp; c < m; c += nw) {
+      const R* a = A + (size_t)c * lda;
+      R s = R(0);
+      for (int i = lane; i < n; i += 32) s += a[i] * a[i];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) taken[c] = 0;
+      key = max(key, cut_key(s, c));
+    }
+    if (lane == 0) keys[warp] = key;
+  }
+  const int q = n < m ? n : m;
+  R d02 = R(0), dk2 = R(0);
+  int j = 0;
+  left = R(0);
+  for (; j < q; ++j) {
+    tm.sync();
+    const unsigned key = cut_best_key(keys + (j & 1) * nw, nw, lane);
+    if (key == 0u) {
+      left = R(0);
+      break;
+    }
+    const int p = (int)(kCutColMask - (key & kCutColMask));
+    const R* ap = A + (size_t)p * lda;
+    R d2 = R(0);
+    for (int i = j + lane; i < n; i += 32) d2 += ap[i] * ap[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+    if (j == 0) d02 = d2;
+    if (j < k) dk2 = d2;
+    left = d02 > R(0) ? d2 / d02 : R(0);
+    if (!(d2 > R(0)) || d2 <= rel2 * dk2 || d2 <= abs2 * d02 || j >= most) break;
+    const R x0 = ap[j], nrm = sqrt(d2);
+    const R alpha = x0 >= R(0) ? -nrm : nrm;
+    const R v0 = x0 - alpha, tau = R(1) / (d2 + fabs(x0) * nrm);
+    if (vr && tm.tid == 0) {
+      vr[4 * j] = v0;
+      vr[4 * j + 1] = tau;
+      vr[4 * j + 2] = alpha;
+      vr[4 * j + 3] = R(p);
+    }
+    unsigned best = 0u;
+    for (int c0 = warp * CB; c0 < m; c0 += nw * CB) {
+      R dots[CB], top[CB];
+      R* ac[CB];
+      unsigned on = 0u;
+#pragma unroll
+      for (int u = 0; u < CB; ++u) {
+        const int c = c0 + u;
+        const bool o = c < m && c != p && !taken[c < m ? c : 0];
+        on |= (unsigned)o << u;
+        ac[u] = A + (size_t)(o ? c : p) * lda;
+        dots[u] = R(0);
+        top[u] = ac[u][j];
+      }
+      if (on)
+#pragma unroll 2
+        for (int i = j + 1 + lane; i < n; i += 32) {
+          const R v = ap[i];
+#pragma unroll
+          for (int u = 0; u < CB; ++u) dots[u] += v * ac[u][i];
+        }
+      const R dot = cut_warp_sums<CB, R>(dots, lane);
+      R w[CB], ss[CB];
+#pragma unroll
+      for (int u = 0; u < CB; ++u) {
+        w[u] = tau * (__shfl_sync(0xffffffffu, dot, u * (32 / CB)) + v0 * top[u]);
+        ss[u] = R(0);
+      }
+      if (on)
+#pragma unroll 2
+        for (int i = j + 1 + lane; i < n; i += 32) {
+          const R v = ap[i];
+          R x[CB];
+#pragma unroll
+          for (int u = 0; u < CB; ++u) {
+            x[u] = ac[u][i] - w[u] * v;
+            ss[u] += x[u] * x[u];
+          }
+#pragma unroll
+          for (int u = 0; u < CB; ++u)
+            if ((on >> u) & 1u) ac[u][i] = x[u];
+        }
+      // the norms below row j summed afresh: the stop is decided on them
+      const R below = cut_warp_sums<CB, R>(ss, lane);
+#pragma unroll
+      for (int u = 0; u < CB; ++u) {
+        const int c = c0 + u;
+        const R s = __shfl_sync(0xffffffffu, below, u * (32 / CB));
+        const bool o = (on >> u) & 1u;
+        if (lane == 0 && c < m) {
+          const R x = top[u] - w[u] * v0;   // R[j][c]
+          if (L) L[(size_t)j * ldl + c] = o ? x : (c == p ? alpha : R(0));
+          if (o) ac[u][j] = x;
+          if (c == p) taken[c] = 1;
+        }
+        if (o) best = max(best, cut_key(s, c));
+      }
+    }
+    if (lane == 0) keys[((j + 1) & 1) * nw + warp] = best;
+  }
+  tm.sync();
+  return j;
+}
+
+template <typename R>
+struct CutTol;
+template <>
+struct CutTol<float> {   // rotate above ~FP32 rounding; done when a sweep saw nothing above 3e-4
+  static __device__ __forceinline__ float rot2() { return 1e-12f; }
+  static __device__ __forceinline__ float done2() { return 1e-7f; }
+};
+template <>
+struct CutTol<double> {  // as TeamTol<double>; a sweep that saw nothing above 1e-8 leaves 1e-16
+  static __device__ __forceinline__ double rot2() { return 1e-30; }
+  static __device__ __forceinline__ double done2() { return 1e-16; }
+};
+__device__ __forceinline__ void cut_rotation(float al, float be, float ga, float& c, float& s) {
+  const float zeta = __fdividef(be - al, 2.f * ga), w = 1.f + zeta * zeta;
+  const float t = copysignf(__fdividef(1.f, fabsf(zeta) + w * rsqrtf(w)), zeta);
+  c = rsqrtf(1.f + t * t);
+  s = t * c;
+}
+__device__ __forceinline__ void cut_rotation(double al, double be, double ga, double& c, double& s) {
+  const double zeta = (be - al) / (2.0 * ga);
+  const double t = copysign(1.0 / (fabs(zeta) + sqrt(1.0 + zeta * zeta)), zeta);
+  c = rsqrt(1.0 + t * t);
+  s = t * c;
+}
+
+// One-sided Jacobi of the r columns (length m, ldl) of L, without V.  g lanes per pair, one barrier
+// per step; NR > 0: both columns' rows of a lane (at most NR) stay in registers between dot and
+// rotation.  The convergence is quadratic, so the sweep that sees no |cos| above the square root of
+// the tolerance is the last.
+template <typename R, int NR>
+__device__ __noinline__ void cut_jacobi(Team tm, R* L, int ldl, int m, int r, int g, int* flag) {
+  constexpr int N = NR > 0 ? NR : 1;
+  const int ne = r + (r & 1), half = ne / 2, mm = ne - 1;
+  const int ngroups = tm.nt / g;
+  const int grp = tm.tid / g, gl = tm.tid % g;
+  for (int sweep = 0; sweep < 30; ++sweep) {
+    if (tm.tid == 0) *flag = 0;
+    tm.sync();
+    bool more = false;
+    for (int k = 0; k < mm; ++k) {
+      for (int i0 = 0; i0 < half; i0 += ngroups) {
+        const int i = i0 + grp;
+        int p = k + i, q = k - i;   // round-robin pair i of step k (team_rr_pair)
+        p = p >= mm ? p - mm : p;
+        q = q < 0 ? q + mm : q;
+        if (i == 0) q = mm;
+        if (p > q) {
+          const int t = p;
+          p = q;
+          q = t;
+        }
+        const bool active = i < half && q < r;
+        R* ap = L + (size_t)(active ? p : 0) * ldl;
+        R* aq = L + (size_t)(active ? q : 0) * ldl;
+        R x[N], y[N];
+        R al = R(0), be = R(0), ga = R(0);
+        if (NR > 0) {
+#pragma unroll
+          for (int t = 0; t < N; ++t) {
+            const int row = gl + t * g;
+            const bool in = active && row < m;
+            x[t] = in ? ap[row] : R(0);
+            y[t] = in ? aq[row] : R(0);
+          }
+#pragma unroll
+          for (int t = 0; t < N; ++t) {
+            al += x[t] * x[t];
+            be += y[t] * y[t];
+            ga += x[t] * y[t];
+          }
+        } else if (active) {
+#pragma unroll 4
+          for (int row = gl; row < m; row += g) {
+            const R u = ap[row], v = aq[row];
+            al += u * u;
+            be += v * v;
+            ga += u * v;
+          }
+        }
+        for (int o = g >> 1; o > 0; o >>= 1) {
+          al += __shfl_xor_sync(0xffffffffu, al, o);
+          be += __shfl_xor_sync(0xffffffffu, be, o);
+          ga += __shfl_xor_sync(0xffffffffu, ga, o);
+        }
+        const R g2 = ga * ga, ab = al * be;
+        if (active && g2 > CutTol<R>::rot2() * ab) {
+          more |= g2 > CutTol<R>::done2() * ab;
+          R c, s;
+          cut_rotation(al, be, ga, c, s);
+          if (NR > 0) {
+#pragma unroll
+            for (int t = 0; t < N; ++t) {
+              const int row = gl + t * g;
+              if (row < m) {
+                ap[row] = c * x[t] - s * y[t];
+                aq[row] = s * x[t] + c * y[t];
+              }
+            }
+          } else {
+#pragma unroll 4
+            for (int row = gl; row < m; row += g) {
+              const R u = ap[row], v = aq[row];
+              ap[row] = c * u - s * v;
+              aq[row] = s * u + c * v;
+            }
+          }
+        }
+      }
+      tm.sync();
+    }
+    if (more) *flag = 1;
+    tm.sync();
+    const int any = *flag;
+    tm.sync();
+    if (!any) break;
+  }
+}
+
+// Norms of the r columns and their descending order.
+template <typename R>
+__device__ __forceinline__ void cut_order(const Team& tm, const R* L, int ldl, int m, int r, R* sg, int* ord) {
+  const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
+  for (int c = warp; c < r; c += nw) {
+    R s = R(0);
+    for (int i = lane; i < m; i += 32) s += L[(size_t)c * ldl + i] * L[(size_t)c * ldl + i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sg[c] = sqrt(s);
+  }
+  tm.sync();
+  for (int j = tm.tid; j < r; j += tm.nt) {
+    const R v = sg[j];
+    int rank = 0;
+    for (int i = 0; i < r; ++i) rank += (sg[i] > v || (sg[i] == v && i < j)) ? 1 : 0;
+    ord[rank] = j;
+  }
+  tm.sync();
+}
+
+// P[kk][i] = sum_c A[c][i] V[c][kk]  (n x k), KB columns per thread.
+template <int KB>
+__device__ __forceinline__ void cut_av(const Team& tm, const double* A, int lda, int n, int m, const double* V, int k,
+                                       double* P) {
+  const int nb = (k + KB - 1) / KB;
+  for (int w = tm.tid; w < n * nb; w += tm.nt) {
+    const int i = w % n, k0 = (w / n) * KB;
+    int kx[KB];
+    double acc[KB];
+#pragma unroll
+    for (int u = 0; u < KB; ++u) {
+      kx[u] = k0 + u < k ? k0 + u : k - 1;
+      acc[u] = 0.0;
+    }
+#pragma unroll 4
+    for (int c = 0; c < m; ++c) {
+      const double a = A[(size_t)c * lda + i];
+#pragma unroll
+      for (int u = 0; u < KB; ++u) acc[u] += a * V[c * k + kx[u]];
+    }
+#pragma unroll
+    for (int u = 0; u < KB; ++u)
+      if (k0 + u < k) P[(size_t)(k0 + u) * n + i] = acc[u];
+  }
+}
+
+// C[kk][c] = sum_i A[c][i] P[kk][i]  (m x k), KB columns per thread.
+template <int KB>
+__device__ __forceinline__ void cut_atp(const Team& tm, const double* A, int lda, int n, int m, const double* P, int k,
+                                        double* C) {
+  const int nb = (k + KB - 1) / KB;
+  for (int w = tm.tid; w < m * nb; w += tm.nt) {
+    const int c = w % m, k0 = (w / m) * KB;
+    const double* a = A + (size_t)c * lda;
+    const double* pk[KB];
+    double acc[KB];
+#pragma unroll
+    for (int u = 0; u < KB; ++u) {
+      pk[u] = P + (size_t)(k0 + u < k ? k0 + u : k - 1) * n;
+      acc[u] = 0.0;
+    }
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+      const double x = a[i];
+#pragma unroll
+      for (int u = 0; u < KB; ++u) acc[u] += x * pk[u][i];
+    }
+#pragma unroll
+    for (int u = 0; u < KB; ++u)
+      if (k0 + u < k) C[(size_t)(k0 + u) * m + c] = acc[u];
+  }
+}
+
+// Columns per thread: as many as leave every thread a task (fewer loads per FMA).
+static __device__ __noinline__ void cut_mul_av(Team tm, const double* A, int lda, int n, int m, const double* V, int k,
+                                               double* P) {
+  if (n * ((k + 3) / 4) >= tm.nt) cut_av<4>(tm, A, lda, n, m, V, k, P);
+  else if (n * ((k + 1) / 2) >= tm.nt) cut_av<2>(tm, A, lda, n, m, V, k, P);
+  else cut_av<1>(tm, A, lda, n, m, V, k, P);
+  tm.sync();
+}
+static __device__ __noinline__ void cut_mul_atp(Team tm, const double* A, int lda, int n, int m, const double* P, int k,
+                                                double* C) {
+  if (m * ((k + 3) / 4) >= tm.nt) cut_atp<4>(tm, A, lda, n, m, P, k, C);
+  else if (m * ((k + 1) / 2) >= tm.nt) cut_atp<2>(tm, A, lda, n, m, P, k, C);
+  else cut_atp<1>(tm, A, lda, n, m, P, k, C);
+  tm.sync();
+}
+
+// V2 = V (3I - V^T V) / 2  (m x k, row-major; S scratch): orthonormal to e^2 from e.
+static __device__ __noinline__ void cut_orthonormalise(Team tm, const double* V, double* V2, double* S, int m, int k) {
+  // four lanes per entry of V^T V
+  for (int w0 = 0; w0 < k * k; w0 += tm.nt / 4) {
+    const int w = w0 + tm.tid / 4, part = tm.tid & 3;
+    const int a = w / k, b = w % k;
+    double s = 0.0;
+    if (w < k * k && a <= b)
+      for (int c = part; c < m; c += 4) s += V[c * k + a] * V[c * k + b];
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    if (w < k * k && a <= b && part == 0) {
+      const double t = (a == b ? 1.5 : 0.0) - 0.5 * s;
+      S[a * k + b] = t;
+      S[b * k + a] = t;
+    }
+  }
+  tm.sync();
+  for (int w = tm.tid; w < m * k; w += tm.nt) {
+    const int c = w / k, b = w % k;
+    double s = 0.0;
+    for (int a = 0; a < k; ++a) s += V[c * k + a] * S[a * k + b];
+    V2[w] = s;
+  }
+  tm.sync();
+}
+
+// Leading dimension of the columns that cut_jacobi turns: = lanes per pair mod 32 at full rank, which
+// puts the lane groups of consecutive pairs on different banks.
+__host__ __device__ __forceinline__ int cut_ldl(int nt, int m) { return bank_ld32(m, team_svd_group(nt, m, m)); }
+
+// Scratch of a cut.  Shared memory takes the small arrays, then the FP32 columns and the vectors.
+struct CutBuf {
+  double *V, *V2;   // [m][k]
+  double* C;        // [k][m]
+  double* P;        // [k][n]
+  float* E;         // [k][m]
+  float* W;         // [q][k]
+  double* S;        // [k][k]
+  double* th;       // [k] theta_j, then [k] 1 / theta_j
+  float* sg;        // [q] singular values (FP32, of the scaled matrix)
+  int* ord;         // [q] descending order
+  float* vcol;      // [n + 34] reflector (n rounded up to 32, and two values)
+  unsigned char* taken;   // [max(m, n)]
+  unsigned* keys;   // [64]
+  static __host__ __device__ int64_t small_bytes(int m, int n, int k) {
+    const int q = m < n ? m : n, x = m < n ? n : m;
+    return (16 * (int64_t)k + 4 * (2 * (int64_t)q + n + 34 + 64) + x + 31) / 16 * 16;
+  }
+  static __host__ __device__ int64_t vec_bytes(int m, int n, int k, bool with_P) {
+    const int q = m < n ? m : n;
+    return (8 * (3 * (int64_t)m * k + (int64_t)k * k + (with_P ? (int64_t)k * n : 0)) + 4 * ((int64_t)m * k + (int64_t)q * k) +
+            31) / 16 * 16;
+  }
+  __device__ void carve_small(unsigned char* base, int m, int n, int k) {
+    const int q = m < n ? m : n;
+    th = reinterpret_cast<double*>(base);
+    sg = reinterpret_cast<float*>(th + 2 * k);
+    ord = reinterpret_cast<int*>(sg + q);
+    vcol = reinterpret_cast<float*>(ord + q);
+    keys = reinterpret_cast<unsigned*>(vcol + n + 34);
+    taken = reinterpret_cast<unsigned char*>(keys + 64);
+  }
+  // P_ == null: P after the other vectors
+  __device__ void carve_vec(double* base, int m, int n, int k, double* P_) {
+    V = base;
+    V2 = V + (size_t)m * k;
+    C = V2 + (size_t)m * k;
+    S = C + (size_t)m * k;
+    double* e = S + (size_t)k * k;
+    P = P_;
+    if (!P_) {
+      P = e;
+      e += (size_t)k * n;
+    }
+    E = reinterpret_cast<float*>(e);
+    W = E + (size_t)m * k;
+  }
+};
+
+// FP32 QR and Jacobi of step 1 and 2 (file comment).  cap floats at Ls (shared) take the columns when
+// they fit -- the rank decides how many are needed, so a rank beyond them starts over with L_g.
+// Returns the rank; the columns are at *L_out.
+__device__ __forceinline__ int cut_fp32(const Team& tm, const double* A, int lda, int n, int m, int k, int expo, float* A_g,
+                                        float* L_g, float* Ls, int cap, CutBuf& b, int* slots, float** L_out, int* ldl_out) {
+  const int q = n < m ? n : m, nw = tm.nt >> 5;
+  const int ldl = cut_ldl(tm.nt, m);
+  const int cols = cap / ldl < q ? cap / ldl : q;
+  const int cpw = (m + nw - 1) / nw;
+  float* L = cols > k ? Ls : L_g;
+  int r = 0;
+  for (int most = cols > k ? cols : q;; most = q, L = L_g) {
+    // the copy in registers: 32 a thread, 64 in the 512-thread blocks (which have 128)
+    if (cpw <= 4 && n <= 128)
+      r = cut_qrcp_reg<4, 4>(tm, A, lda, n, m, k, expo, 1e-6f, 1e-12f, most, L, ldl, b.vcol, b.keys);
+    else if (cpw <= 8 && n <= 128)
+      r = cut_qrcp_reg<8, 4>(tm, A, lda, n, m, k, expo, 1e-6f, 1e-12f, most, L, ldl, b.vcol, b.keys);
+    else if (cpw <= 4 && n <= 256)
+      r = cut_qrcp_reg<4, 8>(tm, A, lda, n, m, k, expo, 1e-6f, 1e-12f, most, L, ldl, b.vcol, b.keys);
+    else if (tm.nt == 512 && cpw <= 8 && n <= 256)
+      r = cut_qrcp_reg<8, 8>(tm, A, lda, n, m, k, expo, 1e-6f, 1e-12f, most, L, ldl, b.vcol, b.keys);
+    else {
+      const int lane = tm.tid & 31;
+      for (int c = tm.tid >> 5; c < m; c += nw)
+        for (int i = lane; i < n; i += 32) A_g[(size_t)c * n + i] = cut_f32(A[(size_t)c * lda + i], expo);
+      tm.sync();
+      float left;
+      r = cut_qrcp<float>(tm, A_g, n, n, m, k, 1e-6f, 1e-12f, most, L, ldl, nullptr, b.taken, b.keys, left);
+    }
+    if (r < most || most == q) break;
+  }
+  *L_out = L;
+  *ldl_out = ldl;
+  if (r <= k) return r;
+  const int g = team_svd_group(tm.nt, m, r), rows = (m + g - 1) / g;
+  if (rows <= 4) cut_jacobi<float, 4>(tm, L, ldl, m, r, g, slots);
+  else if (rows <= 8) cut_jacobi<float, 8>(tm, L, ldl, m, r, g, slots);
+  else if (rows <= 16) cut_jacobi<float, 16>(tm, L, ldl, m, r, g, slots);
+  else cut_jacobi<float, 0>(tm, L, ldl, m, r, g, slots);
+  cut_order<float>(tm, L, ldl, m, r, b.sg, b.ord);
+  return r;
+}
+
+// See the file comment.  2^expo: the magnitude of A's largest entry.  b.P receives the carry
+// U_k^T M, b.V the vectors; slots: two shared ints.  Returns false (nothing usable) when the cut is not
+// one for this path; *r32 is then the FP32 rank.
+static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, int n, int m, int k, int expo, float* A_g,
+                                             float* L_g, float* Ls, int cap, CutBuf& b, int* slots, double* s0, int* r32) {
+  const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
+  float* L;
+  int ldl;
+  const int r = cut_fp32(tm, A, lda, n, m, k, expo, A_g, L_g, Ls, cap, b, slots, &L, &ldl);
+  *r32 = r;
+  if (r <= k) return false;
+  {
+    // FP32 knows the values to ~1e-7 of the largest: the gap has to be clear of that and of the
+    // multiplet rule
+    const float t0 = b.sg[b.ord[0]], tk = b.sg[b.ord[k - 1]], tn = b.sg[b.ord[k]];
+    if (!(tk >= 1e-5f * t0) || !(tk - tn > 1e-4f * tk) || !(tk - tn > 1e-6f * t0)) return false;
+  }
+  double *V = b.V, *V2 = b.V2;
+  for (int w = tm.tid; w < m * k; w += tm.nt) {
+    const int c = w / k, o = b.ord[w % k];
+    V[w] = double(L[(size_t)o * ldl + c] / b.sg[o]);
+  }
+  tm.sync();
+  const double unit2 = ldexp(1.0, -2 * expo);
+  float prev = 0.f;
+  bool ok = false, last = false;
+  for (int it = 0; it < 10; ++it) {
+    cut_orthonormalise(tm, V, V2, b.S, m, k);
+    {
+      double* t = V;
+      V = V2;
+      V2 = t;
+    }
+    cut_mul_av(tm, A, lda, n, m, V, k, b.P);
+    if (last) {
+      ok = true;
+      break;
+    }
+    if (tm.tid == 0) slots[1] = 0;
+    cut_mul_atp(tm, A, lda, n, m, b.P, k, b.C);
+    for (int w0 = 0; w0 < k * k; w0 += tm.nt / 4) {   // S = V^T C, four lanes per entry
+      const int w = w0 + tm.tid / 4, part = tm.tid & 3;
+      const int a = w / k, j = w % k;
+      double s = 0.0;
+      if (w < k * k)
+        for (int c = part; c < m; c += 4) s += V[c * k + a] * b.C[(size_t)j * m + c];
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      if (w < k * k && part == 0) {
+        b.S[w] = s;
+        if (a == j) {
+          b.th[j] = s;
+          b.th[k + j] = 1.0 / s;
+        }
+      }
+    }
+    tm.sync();
+    float worst = 0.f;
+    const float it0 = float(b.th[k]);
+    for (int w = tm.tid; w < m * k; w += tm.nt) {
+      const int j = w / m, c = w % m;
+      double s = b.C[w];
+      for (int a = 0; a < k; ++a) s -= V[c * k + a] * b.S[a * k + j];
+      const float e = float(s * b.th[k + j]);
+      b.E[w] = e;
+      worst = fmaxf(worst, fabsf(e) * sqrtf(float(b.th[j]) * it0));
+    }
+    const unsigned wb = __reduce_max_sync(0xffffffffu, __float_as_uint(worst));
+    if (lane == 0) atomicMax(slots + 1, (int)wb);
+    tm.sync();
+    const float res = __int_as_float(slots[1]);
+    // converged: the residual at FP64 rounding (or no longer falling just above it)
+    if (res <= 5e-16f || (it > 0 && res <= 2e-14f && res > 0.1f * prev)) {
+      ok = true;
+      break;
+    }
+    if (!(res < 1e-2f) || (it > 0 && !(res < 0.3f * prev))) break;
+    for (int i = warp; i < r - k; i += nw) {   // (v_i . e_j) rho / (1 - rho) / sigma_i, a warp per i
+      const int o = b.ord[k + i];
+      const float* l = L + (size_t)o * ldl;
+      const float s2 = b.sg[o] * b.sg[o];
+      for (int j0 = 0; j0 < k; j0 += 4) {
+        float d[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int c = lane; c < m; c += 32) {
+          const float x = l[c];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) d[u] += x * b.E[(size_t)(j0 + u < k ? j0 + u : k - 1) * m + c];
+        }
+        const float mine = cut_warp_sums<4, float>(d, lane);
+        const int j = j0 + (lane >> 3);
+        if ((lane & 7) == 0 && j < k) {
+          const float rho = s2 / float(b.th[j] * unit2);
+          b.W[(size_t)i * k + j] = mine / s2 * (rho / (1.f - rho));
+        }
+      }
+    }
+    tm.sync();
+    for (int w = tm.tid; w < m * k; w += tm.nt) {
+      const int j = w / m, c = w % m;
+      float t = b.E[w];
+#pragma unroll 4
+      for (int i = 0; i < r - k; ++i) t += L[(size_t)b.ord[k + i] * ldl + c] * b.W[(size_t)i * k + j];
+      V[c * k + j] += double(t);
+    }
+    // the pass gained a factor res / prev; the next residual is predicted below rounding
+    last = it > 0 && res * (res / prev) * 8.f < 5e-16f;
+    prev = res;
+    tm.sync();
+  }
+  b.V = V;
+  if (ok) *s0 = sqrt(b.th[0]);
+  return ok;
+}
+
+// Cut of rank <= most (nothing to truncate): X = M (n columns of length m, column-major, ld m;
+// destroyed); U (m x r) into An (row-major), the carry R (r x n) into Cn; Qs: most x m scratch, vr:
+// 4 most, all FP64.  Returns r, or -1 when more than `most` pivots lie above the cutoff.  *rest: the
+// largest squared column norm left out over the largest of all.
+static __device__ __noinline__ int cut_rank(Team tm, double* X, int m, int n, int most, double cutoff, double* An, double* Cn,
+                                            double* Qs, double* vr, CutBuf& b, double* s0, double* rest) {
+  double left;
+  const int q = m < n ? m : n;
+  const int r = cut_qrcp<double>(tm, X, m, m, n, 0, 0.0, cutoff * cutoff, most < q ? most : q, nullptr, 0, vr, b.taken,
+                                 b.keys, left);
+  if (r == 0 || (r < q && left > cutoff * cutoff)) return -1;
+  const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
+  for (int kk = warp; kk < r; kk += nw) {   // Q e_kk = H_0 ... H_kk e_kk, a warp per column
+    double* x = Qs + (size_t)kk * m;
+    for (int i = lane; i < m; i += 32) x[i] = i == kk ? 1.0 : 0.0;
+    for (int j = kk; j >= 0; --j) {   // a lane's rows are its own: no exchange but the dot product
+      const double v0 = vr[4 * j], tau = vr[4 * j + 1];
+      const double* v = X + (size_t)(int)vr[4 * j + 3] * m;
+      double w = 0.0;
+      for (int i = lane; i < m; i += 32)
+        if (i >= j) w += (i == j ? v0 : v[i]) * x[i];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+      w *= tau;
+      for (int i = lane; i < m; i += 32)
+        if (i >= j) x[i] -= w * (i == j ? v0 : v[i]);
+    }
+  }
+  for (int w = tm.tid; w < r * n; w += tm.nt) Cn[w] = X[(size_t)(w % n) * m + w / n];
+  tm.sync();
+  for (int w = tm.tid; w < r * r; w += tm.nt) {   // pivot columns: alpha on the diagonal, zero below it
+    const int j = w / r, i = w % r;
+    if (i >= j) Cn[(size_t)i * n + (int)vr[4 * j + 3]] = i == j ? vr[4 * j + 2] : 0.0;
+  }
+  for (int w = tm.tid; w < m * r; w += tm.nt) An[w] = Qs[(size_t)(w % r) * m + w / r];
+  *s0 = fabs(vr[2]);
+  *rest = r < q ? left : 0.0;
+  tm.sync();
+  return r;
+}
+
+// Any cut, in FP64: pivoted QR of A (X: a copy, ld n; destroyed), Jacobi on R^T (L, ld
+// cut_ldl); sv: 2 min(m, n) singular values (unsorted, then sorted), ord: their
+// order.  Returns the number kept by the rule (0: the matrix is zero or not finite); U into An,
+// the carry into Cn; *rest: the discarded fraction.
+static __device__ __noinline__ int cut_full(Team tm, const double* A, int lda, double* X, int m, int n, int most,
+                                            double cutoff, double rtol, double* L, double* sv, int* ord, double* An,
+                                            double* Cn, CutBuf& b, int* slots, double* s0, double* rest) {
+  const int lane = tm.tid & 31, nw = tm.nt >> 5, q = n < m ? n : m;
+  for (int c = tm.tid >> 5; c < m; c += nw)
+    for (int i = lane; i < n; i += 32) X[(size_t)c * n + i] = A[(size_t)c * lda + i];
+  tm.sync();
+  double left;
+  const int ldl = cut_ldl(tm.nt, m);
+  // directions below 1e-15 of the largest are rounding of A
+  const int r = cut_qrcp<double>(tm, X, n, n, m, 0, 0.0, 1e-30, q, L, ldl, nullptr, b.taken, b.keys, left);
+  if (r == 0) return 0;
+  if (r > 1) {
+    const int g = team_svd_group(tm.nt, m, r);
+    if ((m + g - 1) / g <= 8) cut_jacobi<double, 8>(tm, L, ldl, m, r, g, slots);
+    else cut_jacobi<double, 0>(tm, L, ldl, m, r, g, slots);
+  }
+  cut_order<double>(tm, L, ldl, m, r, sv, ord);
+  double* srt = sv + q;
+  for (int i = tm.tid; i < r; i += tm.nt) srt[i] = sv[ord[i]];
+  tm.sync();
+  *s0 = srt[0];
+  if (!(srt[0] > 0.0)) return 0;
+  if (tm.tid == 0) {
+    slots[0] = team_keep_count<double>(srt, r, most, cutoff, rtol);
+    double tot = 0.0, disc = 0.0;
+    for (int i = 0; i < r; ++i) {
+      tot += srt[i] * srt[i];
+      if (i >= slots[0]) disc += srt[i] * srt[i];
+    }
+    b.th[0] = disc / tot;
+  }
+  tm.sync();
+  const int k = slots[0];
+  *rest = b.th[0];
+  for (int w = tm.tid; w < m * k; w += tm.nt) {
+    const int o = ord[w % k];
+    An[w] = L[(size_t)o * ldl + w / k] / sv[o];
+  }
+  tm.sync();
+  cut_mul_av(tm, A, lda, n, m, An, k, Cn);
+  return k;
+}
+
+}  // namespace td

@@ -12,19 +12,14 @@
 // Arithmetic.  The contraction computes in FP64 on both paths (T is the storage type of the
 // site tensors it reads): the class-parity leg carries both cosets through one MPS, so FP32
 // sums and FP32 singular vectors err by ~eps32 times the majority coset's weight, a relative
-// error of ~eps32 exp(margin) on the minority coset.  Each cut's left singular vectors come
-// from a one-sided Jacobi SVD; when M^T (n x m) has at least as many rows as columns it is
-// first reduced by a Householder QR, M^T = Q R, and the Jacobi orthogonalises the m columns
-// of the m x m factor R (half-length columns; R V has orthogonal columns exactly when M^T V
-// has).  The carry is then (M^T V_k)^T from the unreduced M^T.  On the mixed path the
-// Jacobi of R is preconditioned by an FP32 solve and finished by FP64 sweeps run to
-// convergence (svd_precond), and only for the chi_mps + 2 columns of largest norm, the only
-// ones a cut can keep (and the one after them, for the multiplet rule): the FP64 sweeps rotate
-// just the pairs that involve one of them.  The gradient pass's recorded forward keeps the
-// unreduced Jacobi on M^T (its records are M^T V and V).
+// error of ~eps32 exp(margin) on the minority coset.  The cuts are those of cut.cuh, to FP64
+// accuracy on every path; the gradient pass's recorded forward takes a one-sided Jacobi SVD of
+// M^T with V accumulated (its records are M^T V and V).
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 
+#include "cut.cuh"
 #include "sweep.cuh"
 #include "team.cuh"
 
@@ -93,11 +88,122 @@ __device__ void build_F(const Team& tm, const FinalArgs& fa, int b, int x, int y
   tm.sync();
 }
 
+// The cut of M = MT^T (m x n) by cut.cuh: the left vectors into An, the unscaled
+// carry into Cn.  Returns the number of states kept (0: the matrix is zero), or -1 when the scratch
+// does not hold the paths (the caller then takes the plain Jacobi of the recorded cuts).
+// Scratch: shared memory (`pool` bytes at `sp`) as far as it goes, then the W, Q and R regions.
+static __device__ __noinline__ int cut(Team tm, const FinalArgs& fa, const double* MT, int ldm, int m, int n,
+                                       double* work, double* W, double* An, double* Cn, unsigned char* sp, int64_t pool,
+                                       int* slots, double (*sums)[32], double* trunc, double* s0) {
+  const int q = m < n ? m : n, cm = fa.chi_mps, kk = cm < q ? cm : q;
+  const int ex = cut_max_exponent(tm, MT, ldm, n, m, slots) - 1023;
+  if (ex == -1023) return 0;
+  *s0 = ldexp(1.0, ex);
+  if (m == 1) {
+    // one state (outside the occupied grid): U = 1, carry = M
+    for (int w = tm.tid; w < n; w += tm.nt) Cn[w] = MT[w];
+    if (tm.tid == 0) An[0] = 1.0;
+    return 1;
+  }
+  CutBuf cb;
+  int64_t wleft = fa.W_elems * 8;
+  unsigned char* wp = reinterpret_cast<unsigned char*>(W);
+  const int64_t small = CutBuf::small_bytes(m, n, kk);
+  if (small <= pool) {
+    cb.carve_small(sp, m, n, kk);
+    sp += small;
+    pool -= small;
+  } else if (small <= wleft) {
+    cb.carve_small(wp, m, n, kk);
+    wp += small;
+    wleft -= small;
+  } else {
+    return -1;
+  }
+  double* Q = work + fa.w_Q;
+  double* Rg = work + fa.w_R;
+  const int64_t l_col = 4 * (int64_t)cut_ldl(tm.nt, m);   // bytes of an FP32 column
+  int k = -1, r32 = 0;
+  double rest = 0.0;   // discarded fraction
+  if (q > cm && ex > -400 && ex < 400) {
+    r32 = q;
+    const int64_t vec_p = CutBuf::vec_bytes(m, n, cm, true), vec = CutBuf::vec_bytes(m, n, cm, false);
+    const bool vs = vec_p + l_col * q <= pool;
+    if (vs || vec <= wleft) {
+      if (vs) cb.carve_vec(reinterpret_cast<double*>(sp), m, n, cm, nullptr);
+      else cb.carve_vec(reinterpret_cast<double*>(wp), m, n, cm, Cn);
+      unsigned char* lp = vs ? sp + vec_p : sp;
+      const int64_t cap = (vs ? pool - vec_p : pool) / 4;
+      if (cut_topk(tm, MT, ldm, n, m, cm, ex, reinterpret_cast<float*>(Q), reinterpret_cast<float*>(Rg),
+                   reinterpret_cast<float*>(lp), (int)cap, cb, slots, s0, &r32)) {
+        k = cm;
+        for (int w = tm.tid; w < m * k; w += tm.nt) An[w] = cb.V[w];
+        if (vs)
+          for (int w = tm.tid; w < k * n; w += tm.nt) Cn[w] = cb.P[w];
+        if (fa.stats) {   // |M - U U^T M|^2 over |M|^2, entry by entry (no cancellation)
+          double disc = 0.0, tot = 0.0;
+          for (int w = tm.tid; w < m * n; w += tm.nt) {
+            const int c = w / n, i = w % n;
+            const double a = MT[(size_t)c * ldm + i];
+            double d = a;
+            for (int j = 0; j < k; ++j) d -= cb.P[(size_t)j * n + i] * cb.V[c * k + j];
+            disc += d * d;
+            tot += a * a;
+          }
+          for (int o = 16; o > 0; o >>= 1) {
+            disc += __shfl_xor_sync(0xffffffffu, disc, o);
+            tot += __shfl_xor_sync(0xffffffffu, tot, o);
+          }
+          if ((tm.tid & 31) == 0) {
+            sums[0][tm.tid >> 5] = disc;
+            sums[1][tm.tid >> 5] = tot;
+          }
+          tm.sync();
+          disc = tot = 0.0;
+          for (int w = 0; w < tm.nt / 32; ++w) {
+            disc += sums[0][w];
+            tot += sums[1][w];
+          }
+          rest = disc / tot;
+        }
+      }
+    }
+  }
+  if (k < 0 && r32 <= cm) {
+    const int64_t need_v = 8 * (4 * (int64_t)kk), need_q = 8 * (int64_t)kk * m, need_x = 8 * (int64_t)m * n;
+    if (need_v + need_q <= wleft) {
+      const bool xs = need_v + need_q + need_x <= pool;
+      unsigned char* base = xs ? sp : wp;
+      double* vr = reinterpret_cast<double*>(base);
+      double* Qs = vr + 4 * kk;
+      double* X = xs ? Qs + (size_t)kk * m : Q;
+      for (int w = tm.tid; w < m * n; w += tm.nt) X[w] = MT[(size_t)(w % m) * ldm + w / m];
+      tm.sync();
+      k = cut_rank(tm, X, m, n, kk, fa.svd_cutoff, An, Cn, Qs, vr, cb, s0, &rest);
+    }
+  }
+  if (k < 0) {
+    const int64_t need_l = 2 * l_col * q, need_x = 8 * (int64_t)m * n;
+    const bool ls = need_l <= pool, xs = ls && need_l + need_x <= pool;
+    double* L = ls ? reinterpret_cast<double*>(sp) : Rg;
+    double* X = xs ? reinterpret_cast<double*>(sp + need_l) : Q;
+    k = cut_full(tm, MT, ldm, X, m, n, cm, fa.svd_cutoff, fa.multiplet_rtol, L, work + fa.w_s,
+                 reinterpret_cast<int*>(work + fa.w_ord), An, Cn, cb, slots, s0, &rest);
+  }
+  if (k > 0 && fa.stats && tm.tid == 0) {
+    trunc[0] = fmax(trunc[0], rest);
+    trunc[1] += rest;
+  }
+  tm.sync();
+  return k;
+}
+
 // One block per shot.  The work region (site tensor F, T1 / V, M^T, carries) lives in
 // shared memory when it fits, otherwise in the shot's global scratch; the boundary MPS is
 // always in global scratch.
-template <typename T, typename R>
-__global__ void __launch_bounds__(1024) k_final(FinalArgs fa) {
+// NT: threads per block; MINB: resident blocks that the registers are to leave room for.
+template <typename T, typename R, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_final(FinalArgs fa) {
   const int b = blockIdx.x;
   const Team tm{(int)threadIdx.x, (int)blockDim.x, 1};
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -116,8 +222,7 @@ __global__ void __launch_bounds__(1024) k_final(FinalArgs fa) {
   __shared__ R slam[4 * kMaxChi];
   __shared__ double logsum_s;
   __shared__ double trunc_s[2];   // largest and summed discarded fraction of the cuts
-  __shared__ R red_s[2];
-  __shared__ double slot_s;
+  __shared__ double sum_s[2][32];
   const int nx = fa.nx, ny = fa.ny;
   if (tm.tid == 0) { logsum_s = 0.0; trunc_s[0] = 0.0; trunc_s[1] = 0.0; }
   for (int x = tm.tid; x < nx; x += tm.nt) {
@@ -196,79 +301,45 @@ __global__ void __launch_bounds__(1024) k_final(FinalArgs fa) {
       R* An = mps[cur ^ 1] + (int64_t)x * fa.mps_stride;
       R* Cn = Cb[cc ^ 1];
       if (x < nx - 1 && y < ny - 1) {
-        // left singular vectors of M = MT^T: one-sided Jacobi on the m columns of MT, or on
-        // the columns of the triangular factor of MT's QR (see the file comment)
+        int k = -1;   // states kept; -1: by the plain Jacobi below
+        double s0 = 0.0;
+        if constexpr (sizeof(R) == 8) {
+          if (!rs)
+            k = cut(tm, fa, MT, ldm, m, n, work, W, An, Cn, smem_raw + (fa.use_smem ? fa.work_elems * sizeof(R) : 0),
+                    fa.cut_smem, meta + 2, sum_s, trunc_s, &s0);
+        }
         R* V = W;
-        const bool qr = !rs && m >= 2 && n >= m;
-        // a wide cut (n < m: the first row, where the incoming MPS has bond 1) has rank <= n:
-        // one-sided Jacobi on the n columns of M (not the m columns of M^T); the left singular
-        // vectors are M's rotated columns, normalised
-        const bool wide = !rs && n < m;
-        const int nc = wide ? n : m;   // singular values computed
-        R* Mt = work + fa.w_Q;
-        const int ldt = bank_ld32(m, team_svd_group(tm.nt, m, n));
-        int ldvv = ldv;
-        if (wide) {
-          for (int w = tm.tid; w < m * n; w += tm.nt) {
-            const int c = w / m, ju = w % m;
-            Mt[c * ldt + ju] = MT[ju * ldm + c];
-          }
-          tm.sync();
-          ldvv = bank_ld32(n, team_svd_group(tm.nt, m, n));
-          team_svd_onesided<R>(tm, Mt, ldt, m, n, V, ldvv, meta + 7, 40, true);
-          team_col_norms<R>(tm, Mt, ldt, m, n, sv);
-        } else if (qr) {
-          R* Qw = work + fa.w_Q;
-          R* Rk = work + fa.w_R;
-          const int ldr = bank_ld32(m, team_svd_group(tm.nt, m, m));
-          ldvv = bank_ld32(m, team_svd_group(tm.nt, m, m));
-          for (int w = tm.tid; w < m * n; w += tm.nt) Qw[(w / n) * n + w % n] = MT[(w / n) * ldm + w % n];
-          tm.sync();
-          team_qr_r<R>(tm, Qw, n, n, m, red_s);
-          for (int w = tm.tid; w < m * m; w += tm.nt) {
-            const int c = w / m, r = w % m;
-            Rk[c * ldr + r] = (r <= c) ? Qw[c * n + r] : R(0);
-          }
-          tm.sync();
-          if constexpr (sizeof(R) == 8) {
-            if (fa.precond)
-              svd_precond(tm, Rk, ldr, m, m, V, ldvv, work + fa.w_P, work + fa.w_T, meta + 7, &slot_s,
-                          fa.chi_mps + 2 < m ? fa.chi_mps + 2 : 0, sv, ord, true);
-            else
-              team_svd_onesided<R>(tm, Rk, ldr, m, m, V, ldvv, meta + 7, 40, true);
-          } else {
-            team_svd_onesided<R>(tm, Rk, ldr, m, m, V, ldvv, meta + 7, 40, true);
-          }
-          team_col_norms<R>(tm, Rk, ldr, m, m, sv);
-        } else {
+        const bool plain = k < 0;
+        if (plain) {
+          // one-sided Jacobi on the m columns of MT, V accumulated (the reverse sweep's record)
           team_svd_onesided<R>(tm, MT, ldm, n, m, V, ldv, meta + 7, 40, true);
           team_col_norms<R>(tm, MT, ldm, n, m, sv);
-        }
-        team_sort_desc<R>(tm, sv, nc, ord);
-        if (tm.tid == 0) {
-          int k = 0;
-          const R s0 = sv[ord[0]];
-          if (s0 > R(0)) {
-            R* srt = sv + m;   // the second half of the singular-value region
-            const int nsv = m < n ? m : n;
-            for (int i = 0; i < nsv; ++i) srt[i] = sv[ord[i]];
-            k = team_keep_count<R>(srt, nsv, fa.chi_mps, fa.svd_cutoff, fa.multiplet_rtol);
-            if (fa.stats) {   // discarded fraction sum_{i >= k} s_i^2 / sum_i s_i^2
-              double tot = 0.0, disc = 0.0;
-              for (int i = 0; i < nsv; ++i) {
-                const double q = double(srt[i]) * double(srt[i]);
-                tot += q;
-                if (i >= k) disc += q;
+          team_sort_desc<R>(tm, sv, m, ord);
+          if (tm.tid == 0) {
+            int kept = 0;
+            if (sv[ord[0]] > R(0)) {
+              R* srt = sv + m;   // the second half of the singular-value region
+              const int nsv = m < n ? m : n;
+              for (int i = 0; i < nsv; ++i) srt[i] = sv[ord[i]];
+              kept = team_keep_count<R>(srt, nsv, fa.chi_mps, fa.svd_cutoff, fa.multiplet_rtol);
+              if (fa.stats) {   // discarded fraction sum_{i >= k} s_i^2 / sum_i s_i^2
+                double tot = 0.0, disc = 0.0;
+                for (int i = 0; i < nsv; ++i) {
+                  const double q = double(srt[i]) * double(srt[i]);
+                  tot += q;
+                  if (i >= kept) disc += q;
+                }
+                const double f = tot > 0.0 ? disc / tot : 0.0;
+                trunc_s[0] = fmax(trunc_s[0], f);
+                trunc_s[1] += f;
               }
-              const double f = tot > 0.0 ? disc / tot : 0.0;
-              trunc_s[0] = fmax(trunc_s[0], f);
-              trunc_s[1] += f;
             }
+            meta[0] = kept;
           }
-          meta[0] = k;
+          tm.sync();
+          k = meta[0];
+          s0 = double(sv[ord[0]]);
         }
-        tm.sync();
-        const int k = meta[0];
         if constexpr (sizeof(R) == 8) {
           if (rs) {
             const FinRecSlot ly(fa.rec_mC, fa.rec_mA, fa.rec_m, fa.rec_n);
@@ -277,7 +348,7 @@ __global__ void __launch_bounds__(1024) k_final(FinalArgs fa) {
             for (int w = tm.tid; w < m; w += tm.nt) { rs[ly.sv + w] = double(sv[w]); rs[ly.ord + w] = ord[w]; }
             if (tm.tid == 0) {
               int e2r = 0;
-              if (k > 0) frexp(double(sv[ord[0]]), &e2r);
+              if (k > 0) frexp(s0, &e2r);
               rs[9] = m; rs[10] = n; rs[11] = k; rs[12] = e2r;
             }
           }
@@ -291,41 +362,19 @@ __global__ void __launch_bounds__(1024) k_final(FinalArgs fa) {
         } else {
           // exact power-of-two normalisation of the carry (its log to the log-scale)
           int e2 = 0;
-          frexp(double(sv[ord[0]]), &e2);
+          frexp(s0, &e2);
           const R inv0 = R(ldexp(1.0, -e2));
-          if (wide) {
+          if (plain) {
             for (int w = tm.tid; w < m * k; w += tm.nt) {
               const int ju = w / k, kk = w % k;
-              An[w] = Mt[ord[kk] * ldt + ju] / sv[ord[kk]];
+              An[w] = V[ord[kk] * ldv + ju];
             }
-            tm.sync();
-            // carry = (M^T U_k)^T from the unrotated M^T
             for (int w = tm.tid; w < k * n; w += tm.nt) {
               const int kk = w / n, c = w % n;
-              R acc = R(0);
-              for (int j = 0; j < m; ++j) acc += MT[j * ldm + c] * An[j * k + kk];
-              Cn[w] = acc * inv0;
+              Cn[w] = MT[ord[kk] * ldm + c] * inv0;
             }
           } else {
-            for (int w = tm.tid; w < m * k; w += tm.nt) {
-              const int ju = w / k, kk = w % k;
-              An[w] = V[ord[kk] * ldvv + ju];
-            }
-            if (qr) {
-              // carry = (M^T V_k)^T from the unreduced M^T
-              for (int w = tm.tid; w < k * n; w += tm.nt) {
-                const int kk = w / n, c = w % n;
-                const R* vk = V + ord[kk] * ldvv;
-                R acc = R(0);
-                for (int j = 0; j < m; ++j) acc += MT[j * ldm + c] * vk[j];
-                Cn[w] = acc * inv0;
-              }
-            } else {
-              for (int w = tm.tid; w < k * n; w += tm.nt) {
-                const int kk = w / n, c = w % n;
-                Cn[w] = MT[ord[kk] * ldm + c] * inv0;
-              }
-            }
+            for (int w = tm.tid; w < k * n; w += tm.nt) Cn[w] *= inv0;
           }
           if (tm.tid == 0) {
             logsum_s += double(e2) * 0.69314718055994530942;
@@ -451,16 +500,37 @@ __global__ void k_finalize(FinalizeArgs f) {
   if (f.margin) f.margin[gb] = lp[dec] - lp[dec ^ 1];
 }
 
-template <typename T, typename R>
-cudaError_t launch_final(const FinalArgs& f, cudaStream_t st) {
-  size_t smem = 0;
-  if (f.use_smem) {
-    smem = (size_t)f.work_elems * sizeof(R);
-    cudaError_t e = cudaFuncSetAttribute(k_final<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <typename T, typename R, int NT, int MINB>
+static cudaError_t final_launch(const FinalArgs& f, cudaStream_t st) {
+  FinalArgs a = f;
+  // dynamic shared memory: the work region when it fits, then scratch for the cuts -- what the
+  // largest can use, within the share of an SM that leaves room for as many blocks as there are (at
+  // most MINB)
+  int dev = 0, nsm = 1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int64_t wk = f.use_smem ? f.work_elems * (int64_t)sizeof(R) : 0;
+  const int per_sm = std::max(1, std::min(MINB, (f.B + nsm - 1) / nsm));
+  const int64_t room = std::min<int64_t>(f.smem_block, f.smem_sm / per_sm - 1024) - (int64_t)kFinalStaticSmem - wk;
+  const int64_t pool = f.rec ? 0 : std::max<int64_t>(0, std::min<int64_t>(room, f.cut_need)) / 16 * 16;
+  a.cut_smem = (int32_t)pool;
+  const size_t smem = (size_t)(wk + pool);
+  if (smem > 0) {
+    e = cudaFuncSetAttribute(k_final<T, R, NT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_final<T, R><<<f.B, f.threads, smem, st>>>(f);
+  k_final<T, R, NT, MINB><<<f.B, NT, smem, st>>>(a);
   return cudaGetLastError();
+}
+
+template <typename T, typename R>
+cudaError_t launch_final(const FinalArgs& f, cudaStream_t st) {
+  switch (f.threads) {
+    case 256: return final_launch<T, R, 256, 3>(f, st);
+    case 512: return final_launch<T, R, 512, 1>(f, st);
+    default: return final_launch<T, R, 1024, 1>(f, st);
+  }
 }
 
 cudaError_t launch_finalize(const FinalizeArgs& f, cudaStream_t st) {

@@ -54,6 +54,8 @@ __device__ __forceinline__ const Override* vshot_ovr(const VShot* vs, const Over
   return (o->kind == kind && o->target == target) ? o : nullptr;
 }
 
+constexpr size_t kFinalStaticSmem = 8 * 1024;   // bound of k_final's own shared arrays
+
 struct FinalArgs {
   const void* gamma;
   int64_t shot_elems;
@@ -68,9 +70,12 @@ struct FinalArgs {
   int64_t off_work;          // work region in the global scratch (when not in shared memory)
   int64_t work_elems;        // work region size (elements)
   int64_t w_F, w_W, w_MT, w_C0, w_C1, w_s, w_ord;   // offsets inside the work region
-  int64_t w_Q, w_R, w_P, w_T;   // QR copy of M^T, its triangular factor, FP32-preconditioning scratch
-  int32_t precond;           // cut SVDs: FP32-preconditioned FP64 Jacobi (mixed path)
+  int64_t w_Q, w_R;          // scratch of the cuts: a copy of the matrix, the columns of its factor
+  int64_t W_elems;           // size of the W region (elements)
   int32_t use_smem;          // work region in dynamic shared memory
+  int32_t cut_need;          // bytes of shared memory the FP32 half of the largest cut can use
+  int32_t cut_smem;          // bytes of it given to this launch (work region in global memory only)
+  int32_t smem_sm, smem_block;   // shared memory of one SM, largest per block (bytes)
   int32_t threads;           // threads per block (one block per shot)
   int32_t nbonds, chi, nslots, slot;
   int32_t nx, ny, chi_mps;
