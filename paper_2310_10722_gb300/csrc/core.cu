@@ -57,14 +57,6 @@ struct CoreSmem {
   }
 };
 
-__device__ __forceinline__ Team make_team(int team_threads) {
-  Team tm;
-  tm.nt = team_threads;
-  tm.tid = threadIdx.x % team_threads;
-  tm.bar = 1 + threadIdx.x / team_threads;
-  return tm;
-}
-
 // The four Gram blocks of item (gate, shot) in FP64: the sum, in chunk order, of the
 // partial Grams of its row chunks.
 __device__ __forceinline__ void load_gram(const Team& tm, const double* gram, int64_t item, int nchunk, int chi,
@@ -79,13 +71,218 @@ __device__ __forceinline__ void load_gram(const Team& tm, const double* gram, in
   }
 }
 
+// FP64 one-sided Jacobi sweeps (as team_svd_onesided with V given) of the items of one block of four
+// warps in lock step: up to four items of one-warp teams, two of two, one of four.
+//
+// What bounds it: an FP64 instruction holds its warp's scheduler for 64 cycles (and the SM's FP64
+// pipe for 19) however many lanes are active, so the sweeps cost what their warp instructions cost.  A
+// team by itself spends ~93 per step of 8 pairs: 12 for the dot products, 6 for their reduction, ~43
+// for the test and the rotation's angles (division, square roots; the same in the 4 lanes of a pair),
+// 32 to apply it -- also for pairs that do not rotate.  Here one warp computes the angles of all the
+// block's pairs, one pair per lane, and the rotations of the pairs that rotate are spread over all
+// four warps row by row; a pair's three sums are reduced side by side (3 instead of 6 instructions for
+// 4 lanes), or, when a block has fewer items than warps, by different warps.  The same operations in
+// the same order on every value: bit for bit the result of team_svd_onesided.  Measured (core time of
+// a decode, before -> now): rotated d9 chi 8, 1000 shots mixed 178 -> 129 ms, 152 shots FP64 66 -> 47
+// ms; d7 FP64, 48 shots 29.4 -> 18.9 ms; d5, 37 shots 10.1 -> 7.4 ms.
+struct GroupJacobi {
+  double al[32], be[32], ga[32];   // squared norms and inner product of every pair of the step
+  double c[32], s[32];
+  int pq[32];                      // p | q << 8 | valid << 16 | parity of the item's sweep << 17
+  int list[32];                    // slots of the pairs that rotate
+  int cnt;
+  int any[4][2];                   // a rotation in the item's sweep (by the sweep's parity)
+  double *A[4], *V[4];
+  int lda[4], ldv[4], m[4], n[4];
+};
+constexpr int kGroupBar = 15;
+// Items per SM below which a round's blocks take fewer items than they have teams for.  Measured
+// (core time of a decode, ms, at 0 / 4 / 8 / 16 / 32): rotated d5 chi 8, 37 shots 9.7 / 7.4 / 7.4 / 7.4 / 7.4,
+// 300 shots 11.5 / 11.5 / 10.9 / 11.2 / 11.3; rotated d7 FP64, 48 shots 26.2 / 23.0 / 18.9 / 18.9 / 18.9;
+// rotated d9 FP64, 152 shots 47.4 / 47.4 / 47.4 / 50.3 / 59.6.
+constexpr int kCoreSpread = 8;
+
+__device__ __forceinline__ bool group_sync_or(bool p) {
+  int r;
+  __syncwarp();   // the barrier takes whole warps
+  asm volatile(
+      "{\n.reg .pred a, b;\nsetp.ne.s32 a, %1, 0;\nbar.red.or.pred b, %2, 128, a;\nselp.s32 %0, 1, 0, b;\n}\n"
+      : "=r"(r)
+      : "r"((int)p), "n"(kGroupBar)
+      : "memory");
+  return r != 0;
+}
+__device__ __forceinline__ void group_sync() {
+  __syncwarp();
+  asm volatile("bar.sync %0, 128;" ::"n"(kGroupBar) : "memory");
+}
+
+// items: of the block (4, 2 or 1); nt: threads of a team, the first of an item's 128 / items threads;
+// the item's arrays are given by its team's thread 0 (has: it has a matrix to work on).
+__device__ void group_jacobi(GroupJacobi& gj, int items, int nt, bool has, double* A, int lda, int m, int n, double* V,
+                             int ldv, int max_sweeps) {
+  const int gt = threadIdx.x, gw = gt >> 5, lane = gt & 31;
+  const int per = 128 / items, it = gt / per, ti = gt % per;
+  const int subs = per / nt, sub = ti / nt, tid = ti % nt;
+  const int S = nt / 4;   // pair slots per item
+  if (ti == 0) {
+    gj.A[it] = A;
+    gj.V[it] = V;
+    gj.lda[it] = lda;
+    gj.ldv[it] = ldv;
+    gj.m[it] = m;
+    gj.n[it] = has && n >= 2 ? n : 0;
+    gj.any[it][0] = gj.any[it][1] = 0;
+  }
+  if (gt < 32) gj.pq[gt] = 0;
+  if (!group_sync_or(ti == 0 && has && n >= 2)) return;
+  A = gj.A[it];
+  lda = gj.lda[it];
+  m = gj.m[it];
+  n = gj.n[it];
+  bool busy = n > 0;
+  int R = 0;   // rows of the block's largest rotation
+  for (int i = 0; i < items; ++i)
+    if (gj.n[i] > 0) R = max(R, gj.m[i] + gj.n[i]);
+  const int ne = n + (n & 1), half = ne / 2;
+  int g = half > 0 ? nt / half : 1;        // lanes per pair, as team_svd_onesided
+  g = g < 1 ? 1 : (g > 32 ? 32 : team_pow2_floor(g));
+  const int rows_max = m > n ? m : n;
+  while (g > 1 && g > rows_max) g >>= 1;
+  const int grp = tid / g, gl = tid % g;
+  int k = 0, sweep = 0, turn = 0;
+  for (;;) {
+    // the step's inner products
+    if (ti < S) {
+      int p, q;
+      team_rr_pair(k, ti, ne, p, q);
+      gj.pq[it * S + ti] = (busy && ti < half && q < n) ? (p | q << 8 | 1 << 16 | (sweep & 1) << 17) : 0;
+    }
+    if (k == 0 && ti == 0) gj.any[it][(sweep & 1) ^ 1] = 0;   // read before the last barrier
+    if (busy) {
+      int p = 0, q = 0;
+      bool active = grp < half;
+      if (active) {
+        team_rr_pair(k, grp, ne, p, q);
+        active = q < n;
+      }
+      const double* ap_ = A + (size_t)p * lda;
+      const double* aq_ = A + (size_t)q * lda;
+      const int slot = it * S + grp;
+      if (subs == 1) {
+        double al = 0.0, be = 0.0, ga = 0.0;
+        if (active)
+          for (int r = gl; r < m; r += g) {
+            const double ap = ap_[r], aq = aq_[r];
+            al += ap * ap;
+            be += aq * aq;
+            ga += ap * aq;
+          }
+        // sums over the pair's lanes, offsets g/2, g/4, ..., 1: the upper half of the lanes takes be, the
+        // lower al, both ga; from the second level on every lane sums one value
+        if (g >= 2) {
+          const bool up = (gl & (g >> 1)) != 0;
+          const double other = __shfl_xor_sync(0xffffffffu, up ? al : be, g >> 1);
+          const double og = __shfl_xor_sync(0xffffffffu, ga, g >> 1);
+          double v = (up ? be : al) + other;
+          ga += og;
+          if (g >= 4) {
+            const bool up2 = (gl & (g >> 2)) != 0;
+            const double o2 = __shfl_xor_sync(0xffffffffu, up2 ? v : ga, g >> 2);
+            v = (up2 ? ga : v) + o2;
+            for (int o = g >> 3; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (active) {
+              if (gl == 0) gj.al[slot] = v;
+              else if (gl == (g >> 2)) gj.ga[slot] = v;
+              else if (gl == (g >> 1)) gj.be[slot] = v;
+            }
+          } else if (active) {
+            if (up) {
+              gj.be[slot] = v;
+            } else {
+              gj.al[slot] = v;
+              gj.ga[slot] = ga;
+            }
+          }
+        } else if (active) {
+          gj.al[slot] = al;
+          gj.be[slot] = be;
+          gj.ga[slot] = ga;
+        }
+      } else {
+        // spare warps: the sums by different ones (two: al and be | ga; four: one each)
+        for (int f = sub; f < 3; f += subs) {   // f: 0 al, 1 ga, 2 be
+          double v = 0.0;
+          const double* x = f == 2 ? aq_ : ap_;
+          const double* y = f == 0 ? ap_ : aq_;
+          if (active)
+            for (int r = gl; r < m; r += g) v += x[r] * y[r];
+          for (int o = g >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (active && gl == 0) (f == 0 ? gj.al : f == 1 ? gj.ga : gj.be)[slot] = v;
+        }
+      }
+    }
+    group_sync();
+    // angles: one pair per lane, the warps in turn
+    if (gw == turn) {
+      const int pq = gj.pq[lane];
+      double c = 1.0, s = 0.0;
+      bool act = false;
+      if (pq) act = jacobi_rot(gj.al[lane], gj.be[lane], gj.ga[lane], TeamTol<double>::rel(), c, s);
+      const unsigned mask = __ballot_sync(0xffffffffu, act);
+      if (act) {
+        gj.c[lane] = c;
+        gj.s[lane] = s;
+        gj.list[__popc(mask & ((1u << lane) - 1u))] = lane;
+        gj.any[lane / S][(pq >> 17) & 1] = 1;
+      }
+      if (lane == 0) gj.cnt = __popc(mask);
+    }
+    turn = (turn + 1) & 3;
+    group_sync();
+    // rotations: the rows of the pairs that rotate, A's then V's, over the block's threads
+    const int tasks = gj.cnt * R;
+    for (int t = gt; t < tasks; t += 128) {
+      const int e = t / R, r = t - e * R;
+      const int slot = gj.list[e], i = slot / S, pq = gj.pq[slot];
+      const int mi = gj.m[i], p = pq & 255, q = (pq >> 8) & 255;
+      if (r < mi + gj.n[i]) {
+        const bool inA = r < mi;
+        double* base = inA ? gj.A[i] : gj.V[i];
+        const int ld = inA ? gj.lda[i] : gj.ldv[i], row = inA ? r : r - mi;
+        double* xp = base + (size_t)p * ld + row;
+        double* xq = base + (size_t)q * ld + row;
+        const double c = gj.c[slot], s = gj.s[slot];
+        const double ap = *xp, aq = *xq;
+        *xp = c * ap - s * aq;
+        *xq = s * ap + c * aq;
+      }
+    }
+    if (busy && ++k == ne - 1) {
+      const int any = gj.any[it][sweep & 1];
+      k = 0;
+      if (!any || ++sweep == max_sweeps) busy = false;
+    }
+    if (!group_sync_or(busy)) break;
+  }
+}
+
 __global__ void k_core2(SweepArgs a, const GateDesc* __restrict__ gates, const double* __restrict__ gram,
-                        double* __restrict__ tbuf, int S, int n_items, int team_threads, int Dm, int precond) {
+                        double* __restrict__ tbuf, int S, int n_items, int items, int team_threads, int Dm, int precond) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const Team tm = make_team(team_threads);
-  const int team = threadIdx.x / team_threads;
-  const int64_t item = (int64_t)blockIdx.x * (blockDim.x / team_threads) + team;
-  if (item >= n_items) return;
+  __shared__ GroupJacobi gj;
+  // `items` items per block of 128 threads; an item's first team_threads threads are its team, the
+  // rest only help in the group's Jacobi sweeps
+  const int per = 128 / items, team = threadIdx.x / per;
+  const int64_t item = (int64_t)blockIdx.x * items + team;
+  if (item >= n_items || (int)threadIdx.x % per >= team_threads) {
+    group_jacobi(gj, items, team_threads, false, nullptr, 1, 0, 0, nullptr, 1, 40);
+    return;
+  }
+  Team tm;
+  tm.nt = team_threads;
+  tm.tid = threadIdx.x % per;
+  tm.bar = 1 + team;
   CoreSmem sm;
   sm.carve(smem_raw + (size_t)team * CoreSmem::bytes(Dm), Dm);
   const int gi = (int)(item / a.B), b = (int)(item % a.B);
@@ -139,6 +336,7 @@ __global__ void k_core2(SweepArgs a, const GateDesc* __restrict__ gates, const d
     for (int w = tm.tid; w < 4 * chi * chi; w += tm.nt) tout[w] = 0.0;
     for (int w = tm.tid; w < Dn; w += tm.nt) lamg[w] = 0.0;
     if (tm.tid == 0) a.logacc[(int64_t)b * a.nslots + S + gd.bond] = -INFINITY;
+    group_jacobi(gj, items, team_threads, false, nullptr, 1, 0, 0, nullptr, 1, 40);
     return;
   }
   const Override* ov = vshot_ovr(a.vs, a.ovr, a.wave_first, b, kOvrGate, a.gate_base + gi);
@@ -174,7 +372,10 @@ __global__ void k_core2(SweepArgs a, const GateDesc* __restrict__ gates, const d
   if (precond)
     svd_precond(tm, TH, ldt, rA, rB, VV, ldv, FF, TT, meta + 8, slot);
   else
-    team_svd_onesided<double>(tm, TH, ldt, rA, rB, VV, ldv, meta + 8, 40, true);
+    for (int w = tm.tid; w < rB * rB; w += tm.nt) VV[(w / rB) * ldv + (w % rB)] = (w / rB == w % rB) ? 1.0 : 0.0;
+  tm.sync();
+  group_jacobi(gj, items, team_threads, true, TH, ldt, rA, rB, VV, ldv, 40);
+  tm.sync();
   team_col_norms<double>(tm, TH, ldt, rA, rB, sm.sv);
   team_sort_desc<double>(tm, sm.sv, rB, sm.order);
   if (tm.tid == 0) {
@@ -252,32 +453,28 @@ __global__ void k_core2(SweepArgs a, const GateDesc* __restrict__ gates, const d
 }
 
 // ---- launch configuration ---------------------------------------------------------------
-// Team size by bond dimension: small cores get one warp each (8 per block), larger ones a
-// group of warps, so that no block-wide barrier serialises independent gates.  The team is
-// split into four segments of at least Dm lanes for the four Cholesky factorisations.
-static void core_shape(int Dm, int& team_threads, int& teams) {
-  if (Dm <= 8) { team_threads = 32; teams = 8; }
-  else if (Dm <= 16) { team_threads = 64; teams = 2; }
-  else { team_threads = 128; teams = 1; }
-}
-
-size_t core2_smem_bytes(int Dm) {
-  int tt, teams;
-  core_shape(Dm, tt, teams);
-  return (size_t)teams * CoreSmem::bytes(Dm);
-}
+// Blocks of 128 threads.  Team by bond dimension: one warp, two or four (four segments of at least
+// Dm lanes for the four Cholesky factorisations).  Items per block: as many as there are teams when
+// the round fills the chip; fewer when it does not, so that an item has spare warps on the other
+// schedulers and the blocks reach more SMs.
+static int core_team(int Dm) { return Dm <= 8 ? 32 : (Dm <= 16 ? 64 : 128); }
 
 template <typename R>
 cudaError_t launch_core2(const SweepArgs& a, const GateDesc* g, int count, int Dm, const double* gram, double* tbuf,
                          int S, bool precond, cudaStream_t st) {
-  int tt, teams;
-  core_shape(Dm, tt, teams);
+  const int tt = core_team(Dm);
   const int64_t n_items = (int64_t)count * a.B;
-  const size_t smem = (size_t)teams * CoreSmem::bytes(Dm);
-  cudaError_t e = cudaFuncSetAttribute(k_core2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int dev = 0, nsm = 1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const unsigned blocks = (unsigned)((n_items + teams - 1) / teams);
-  k_core2<<<blocks, tt * teams, smem, st>>>(a, g, gram, tbuf, S, (int)n_items, tt, Dm, precond ? 1 : 0);
+  int items = 128 / tt;
+  while (items > 1 && n_items <= (int64_t)kCoreSpread * nsm * items / 4) items /= 2;
+  const size_t smem = (size_t)items * CoreSmem::bytes(Dm);
+  e = cudaFuncSetAttribute(k_core2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const unsigned blocks = (unsigned)((n_items + items - 1) / items);
+  k_core2<<<blocks, 128, smem, st>>>(a, g, gram, tbuf, S, (int)n_items, items, tt, Dm, precond ? 1 : 0);
   return cudaGetLastError();
 }
 

@@ -192,7 +192,6 @@ cudaError_t launch_copy_rows(const double* src, int64_t src_stride, int64_t src_
 template <typename R>
 cudaError_t launch_core2(const SweepArgs& a, const GateDesc* g, int count, int Dm, const double* gram, double* tbuf,
                          int S, bool precond, cudaStream_t st);
-size_t core2_smem_bytes(int Dm);
 
 // Gram and update passes (absorb.cu), one warp per (gate side, shot, chunk of kChunkRows
 // rows); Dm = the round's largest bond dimension (before or after the gate).

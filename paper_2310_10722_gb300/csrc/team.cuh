@@ -52,14 +52,12 @@ struct TeamTol<float> {
 // Pair i of step k of the round-robin ("circle") ordering of ne (even) players; player
 // ne-1 stays in place.  p < q on return.
 __device__ __forceinline__ void team_rr_pair(int k, int i, int ne, int& p, int& q) {
-  const int m = ne - 1;
-  if (i == 0) {
-    p = k;
-    q = m;
-  } else {
-    p = (k + i) % m;
-    q = (k - i + m) % m;
-  }
+  const int m = ne - 1;   // 0 <= k < m, 0 <= i < ne / 2
+  p = k + i;
+  if (p >= m) p -= m;
+  q = k - i;
+  if (q < 0) q += m;
+  if (i == 0) q = m;
   if (p > q) {
     const int t = p;
     p = q;
@@ -236,19 +234,33 @@ __device__ __forceinline__ void team_pchol_rinv4(const Team& tm, const double* R
   tm.sync();
 }
 
+// Comparisons of the Jacobi test on bit patterns where the values are known not to be negative (they
+// order as integers): an FP64 comparison holds the FP64 pipe like a multiplication.  le: a <= b for
+// a, b >= 0 (false when either is NaN, as in floating point).
+__device__ __forceinline__ bool nonneg_le(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  return x <= y && y <= 0x7FF0000000000000ll;
+}
+__device__ __forceinline__ bool nonneg_le(float a, float b) { return a <= b; }
+__device__ __forceinline__ bool is_zero(double a) { return (__double_as_longlong(a) << 1) == 0ll; }
+__device__ __forceinline__ bool is_zero(float a) { return a == 0.f; }
+__device__ __forceinline__ bool below_zero(double a) { return __double_as_longlong(a) < 0ll && !is_zero(a); }
+__device__ __forceinline__ bool below_zero(float a) { return a < 0.f; }
+
 // Rotation (c, s) of the one-sided Jacobi step for columns with squared norms al, be and
 // inner product ga; false when the pair is already orthogonal to working precision
 // (ga^2 <= tol^2 al be), or when a column is negligible (squared norm below tiny(); FP32
 // solves run on matrices scaled to a largest entry of 1).
 template <typename R>
 __device__ __forceinline__ bool jacobi_rot(R al, R be, R ga, R tol, R& c, R& s) {
-  if (ga == R(0) || al <= TeamTol<R>::tiny() || be <= TeamTol<R>::tiny() || ga * ga <= tol * tol * (al * be)) {
+  if (is_zero(ga) || nonneg_le(al, TeamTol<R>::tiny()) || nonneg_le(be, TeamTol<R>::tiny()) ||
+      nonneg_le(ga * ga, tol * tol * (al * be))) {
     c = R(1);
     s = R(0);
     return false;
   }
   const R zeta = (be - al) / (R(2) * ga);
-  const R t = (zeta >= R(0) ? R(1) : R(-1)) / (fabs(zeta) + sqrt(R(1) + zeta * zeta));
+  const R t = (below_zero(zeta) ? R(-1) : R(1)) / (fabs(zeta) + sqrt(R(1) + zeta * zeta));
   c = rsqrt(R(1) + t * t);
   s = t * c;
   return true;
@@ -405,16 +417,20 @@ __device__ __forceinline__ int team_keep_count(const R* s, int n, int chi, doubl
 
 // Max |x| over the m x n column-major matrix x (ld), through a shared double slot.
 __device__ inline double team_absmax(const Team& tm, const double* x, int ld, int m, int n, double* slot) {
-  double v = 0.0;
-  for (int w = tm.tid; w < m * n; w += tm.nt) v = fmax(v, fabs(x[(w / m) * ld + (w % m)]));
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  // on the bit patterns, which order non-negative doubles (an FP64 fmax is two FP64 instructions); a
+  // NaN does not count, as in fmax
+  unsigned long long v = 0ull;
+  for (int w = tm.tid; w < m * n; w += tm.nt) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x[(w / m) * ld + (w % m)]) & 0x7FFFFFFFFFFFFFFFull;
+    v = (u > v && u <= 0x7FF0000000000000ull) ? u : v;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long u = __shfl_xor_sync(0xffffffffu, v, o);
+    v = u > v ? u : v;
+  }
   if (tm.tid == 0) *slot = 0.0;
   tm.sync();
-  if ((tm.tid & 31) == 0) {
-    // benign max via compare-and-swap on the bit pattern (non-negative doubles order as integers)
-    unsigned long long* p = reinterpret_cast<unsigned long long*>(slot);
-    atomicMax(p, (unsigned long long)__double_as_longlong(v));
-  }
+  if ((tm.tid & 31) == 0) atomicMax(reinterpret_cast<unsigned long long*>(slot), v);
   tm.sync();
   const double r = *slot;
   tm.sync();
@@ -433,19 +449,19 @@ __device__ __forceinline__ void team_gemm(const Team& tm, const R* A, int lda, c
   }
 }
 
-// One-sided Jacobi SVD of A (m x n, column-major, lda; as team_svd_onesided) preconditioned
-// by an FP32 solve (mixed-precision Jacobi): the FP32 Jacobi runs on a copy scaled to a
-// largest entry of 1; its right factor, re-orthogonalised in FP64 by one Newton-Schulz step
-// V <- V (3I - V^T V) / 2, is applied to A in FP64, and FP64 Jacobi sweeps then run to
-// convergence from it.  The FP32 solve cannot resolve singular values below ~1e-7 of the
-// largest, so the FP64 sweeps are never cut short.  V column-major (ldv).  F: scratch of
-// >= max(m, n) * (max(m, n) + 1) doubles (it also holds the two FP32 matrices); Tt: >= n*n
-// doubles; flag: one team-shared int; slot: one team-shared double.
+// Start of a one-sided Jacobi SVD of A (m x n, column-major, lda) from an FP32 solve
+// (mixed-precision Jacobi): the FP32 Jacobi runs on a copy scaled to a largest entry of 1; its
+// right factor, re-orthogonalised in FP64 by one Newton-Schulz step V <- V (3I - V^T V) / 2, is applied
+// to A in FP64; FP64 Jacobi sweeps (the caller's, V updated along) then run to convergence from it.
+// The FP32 solve cannot resolve singular values below ~1e-7 of the largest, so the FP64 sweeps are
+// never cut short.  V column-major (ldv).  F: scratch of >= max(m, n) * (max(m, n) + 1) doubles (it
+// also holds the two FP32 matrices); Tt: >= n*n doubles; flag: one team-shared int; slot: one
+// team-shared double.  Not synchronised on return.
 __device__ inline void svd_precond(const Team& tm, double* A, int lda, int m, int n, double* V, int ldv, double* F,
                                    double* Tt, int* flag, double* slot) {
   const double amax = team_absmax(tm, A, lda, m, n, slot);
-  if (!(amax > 0.0) || n < 2) {
-    team_svd_onesided<double>(tm, A, lda, m, n, V, ldv, flag, 40, true);
+  if (!(amax > 0.0) || n < 2) {   // nothing to precondition: V = 1
+    for (int w = tm.tid; w < n * n; w += tm.nt) V[(w / n) * ldv + (w % n)] = (w / n == w % n) ? 1.0 : 0.0;
     return;
   }
   const int la32 = odd_ld(m), lv32 = odd_ld(n);
@@ -467,7 +483,7 @@ __device__ inline void svd_precond(const Team& tm, double* A, int lda, int m, in
   // symmetric: the entries i <= j are computed and mirrored (the same products in the same
   // order, so the mirror is exact)
   for (int w = tm.tid; w < n * (n + 1) / 2; w += tm.nt) {
-    int j = (int)((sqrt(8.0 * w + 1.0) - 1.0) * 0.5);
+    int j = (int)((sqrtf(8.0f * w + 1.0f) - 1.0f) * 0.5f);   // corrected below
     while ((j + 1) * (j + 2) / 2 <= w) ++j;
     while (j * (j + 1) / 2 > w) --j;
     const int i = w - j * (j + 1) / 2;   // 0 <= i <= j
@@ -498,7 +514,6 @@ __device__ inline void svd_precond(const Team& tm, double* A, int lda, int m, in
   }
   tm.sync();
   for (int w = tm.tid; w < m * n; w += tm.nt) A[(w / m) * lda + (w % m)] = F[w];
-  team_svd_onesided<double>(tm, A, lda, m, n, V, ldv, flag, 40, false);
 }
 
 }  // namespace td
