@@ -231,7 +231,7 @@ static void final_layout(td_network* net, int threads, bool allow_smem = true) {
     // the largest cut that truncates: small arrays, vectors and FP32 columns
     const int m_max = cm * Dm, n_max = (int)(cmx * Dm * 2);
     const int64_t need = td::CutBuf::small_bytes(m_max, n_max, cm) + td::CutBuf::vec_bytes(m_max, n_max, cm, true) +
-                         4 * (int64_t)td::cut_ldl(threads, m_max) * m_max;
+                         4 * (int64_t)td::cut_ld32(threads, m_max) * m_max;
     net->fin.cut_need = (int32_t)std::min<int64_t>(need, 1 << 30);
     net->fin.smem_sm = net->smem_sm;
     net->fin.smem_block = net->smem_optin;

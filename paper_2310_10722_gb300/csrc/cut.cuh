@@ -97,43 +97,58 @@ __device__ __forceinline__ unsigned cut_best_key(const unsigned* keys, int nw, i
   return __reduce_max_sync(0xffffffffu, lane < nw ? keys[lane] : 0u);
 }
 
+// Two FP32 values in a 64-bit register: one instruction for both (FFMA2).
+__device__ __forceinline__ uint64_t f2_pack(float lo, float hi) {
+  return (uint64_t)__float_as_uint(lo) | ((uint64_t)__float_as_uint(hi) << 32);
+}
+__device__ __forceinline__ float f2_lo(uint64_t v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float f2_hi(uint64_t v) { return __uint_as_float((unsigned)(v >> 32)); }
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
 // Householder QR with column pivoting of the FP32 copy of A (n x m FP64, scaled by 2^-expo), the
 // copy in registers: warp w holds columns w, w + nw, ... (CPW of them), a lane rows lane + 32 t
-// (t < RPL).  Two barriers per step: the pivot is known after the first, its column (written by its
-// warp) after the second; dot products and norms of a warp's columns are reduced together.  The norm
-// of a column after step j is its norm before it, summed afresh, minus R[j][c]^2.  Stops at the
-// first pivot norm^2 <= max(rel2 * (that of the k-th pivot), abs2 * (that of the first)) or after
-// `most` steps; L[j * ldl + c] = R[j][c].  vcol: n rounded up to 32, + 2 floats; keys: nw.
-// Measured (64 x 128, 256 threads): see DESIGN; the version with the copy in memory took 10x.
+// (t < RPL, two per register); rows that are done are zeroed there, so nothing is masked.  Two barriers
+// per step: the pivot is known after the first, its column (written by its warp) after the second;
+// dot products and norms of a warp's columns are reduced together.  The norm of a column after step j
+// is its norm before it, summed afresh, minus R[j][c]^2.  Stops at the first pivot norm^2 <=
+// max(rel2 * (that of the k-th pivot), abs2 * (that of the first)) or after `most` steps;
+// L[j * ldl + c] = R[j][c].  vcol: n rounded up to 32, + 2 floats; keys: nw.
 template <int CPW, int RPL>
 __device__ __noinline__ int cut_qrcp_reg(Team tm, const double* A, int lda, int n, int m, int k, int expo, float rel2,
                                          float abs2, int most, float* L, int ldl, float* vcol, unsigned* keys) {
+  constexpr int H = RPL / 2;
   const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
-  float a[CPW][RPL];
-  unsigned taken = 0u;
+  uint64_t a[CPW][H];
+  unsigned taken = 0u, key0 = 0u;
 #pragma unroll
   for (int u = 0; u < CPW; ++u) {
     const int c = warp + u * nw;
     if (c >= m) taken |= 1u << u;
+    uint64_t s2 = 0ull;
 #pragma unroll
-    for (int t = 0; t < RPL; ++t) {
-      const int i = lane + 32 * t;
-      a[u][t] = (c < m && i < n) ? cut_f32(A[(size_t)c * lda + i], expo) : 0.f;
+    for (int t = 0; t < H; ++t) {
+      const int i = lane + 64 * t;
+      const double* col = A + (size_t)(c < m ? c : 0) * lda;
+      const float lo = (c < m && i < n) ? cut_f32(col[i], expo) : 0.f;
+      const float hi = (c < m && i + 32 < n) ? cut_f32(col[i + 32], expo) : 0.f;
+      a[u][t] = f2_pack(lo, hi);
+      s2 = f2_fma(a[u][t], a[u][t], s2);
     }
+    float s = f2_lo(s2) + f2_hi(s2);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (c < m) key0 = max(key0, cut_key(s, c));
   }
-  {
-    unsigned key = 0u;
-#pragma unroll
-    for (int u = 0; u < CPW; ++u) {
-      float s = 0.f;
-#pragma unroll
-      for (int t = 0; t < RPL; ++t) s += a[u][t] * a[u][t];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (!((taken >> u) & 1u)) key = max(key, cut_key(s, warp + u * nw));
-    }
-    if (lane == 0) keys[warp] = key;
-  }
+  if (lane == 0) keys[warp] = key0;
   const int q = n < m ? n : m, nv = (n + 31) & ~31;
   float d02 = 0.f, dk2 = 0.f;
   int j = 0;
@@ -145,49 +160,55 @@ __device__ __noinline__ int cut_qrcp_reg(Team tm, const double* A, int lda, int 
     if (j == 0) d02 = g2;
     if (j < k) dk2 = g2;
     if (key == 0u || !(g2 > 0.f) || g2 <= rel2 * dk2 || g2 <= abs2 * d02) break;
+    const int jl = j & 31, jt = j >> 6;
+    const bool jh = (j >> 5) & 1;
     if (warp == p % nw) {   // the pivot column becomes the reflector
       const int pu = p / nw;
-      float x[RPL], s = 0.f, x0 = 0.f;
+      uint64_t x[H], s2 = 0ull;
+      float x0 = 0.f;
 #pragma unroll
-      for (int t = 0; t < RPL; ++t) {
-        x[t] = 0.f;
+      for (int t = 0; t < H; ++t) {
+        x[t] = 0ull;
 #pragma unroll
         for (int u = 0; u < CPW; ++u) x[t] = u == pu ? a[u][t] : x[t];
-        const int i = lane + 32 * t;
-        if (i < j) x[t] = 0.f;
-        s += x[t] * x[t];
-        if (i == j) x0 = x[t];
+        s2 = f2_fma(x[t], x[t], s2);
+        if (t == jt) x0 = jh ? f2_hi(x[t]) : f2_lo(x[t]);
       }
+      float s = f2_lo(s2) + f2_hi(s2);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      x0 = __shfl_sync(0xffffffffu, x0, j & 31);
-      const float nrm = sqrtf(s), alpha = x0 >= 0.f ? -nrm : nrm;
+      x0 = __shfl_sync(0xffffffffu, x0, jl);
+      const float nrm = s * rsqrtf(fmaxf(s, 1e-37f)), alpha = x0 >= 0.f ? -nrm : nrm;
 #pragma unroll
-      for (int t = 0; t < RPL; ++t) {
-        const int i = lane + 32 * t;
-        if (i < nv) vcol[i] = i == j ? x0 - alpha : x[t];
+      for (int t = 0; t < H; ++t) {
+        const int i = lane + 64 * t;
+        if (i < nv) vcol[i] = i == j ? x0 - alpha : f2_lo(x[t]);
+        if (i + 32 < nv) vcol[i + 32] = i + 32 == j ? x0 - alpha : f2_hi(x[t]);
       }
       if (lane == 0) {
-        vcol[nv] = s > 0.f ? 1.f / (s + fabsf(x0) * nrm) : 0.f;   // 2 / v.v
+        vcol[nv] = s > 0.f ? __fdividef(1.f, s + fabsf(x0) * nrm) : 0.f;   // 2 / v.v
         vcol[nv + 1] = alpha;
       }
     }
     tm.sync();
-    float v[RPL];
+    uint64_t v[H];
 #pragma unroll
-    for (int t = 0; t < RPL; ++t) v[t] = lane + 32 * t < nv ? vcol[lane + 32 * t] : 0.f;
+    for (int t = 0; t < H; ++t) {
+      const int i = lane + 64 * t;
+      v[t] = f2_pack(i < nv ? vcol[i] : 0.f, i + 32 < nv ? vcol[i + 32] : 0.f);
+    }
     const float tau = vcol[nv], alpha = vcol[nv + 1];
     float sums[2 * CPW];
 #pragma unroll
     for (int u = 0; u < CPW; ++u) {
-      sums[u] = 0.f;
-      sums[CPW + u] = 0.f;
+      uint64_t d = 0ull, s2 = 0ull;
 #pragma unroll
-      for (int t = 0; t < RPL; ++t) {
-        sums[u] += v[t] * a[u][t];
-        const float x = lane + 32 * t < j ? 0.f : a[u][t];
-        sums[CPW + u] += x * x;
+      for (int t = 0; t < H; ++t) {
+        d = f2_fma(v[t], a[u][t], d);
+        s2 = f2_fma(a[u][t], a[u][t], s2);
       }
+      sums[u] = f2_lo(d) + f2_hi(d);
+      sums[CPW + u] = f2_lo(s2) + f2_hi(s2);
     }
     const float mine = cut_warp_sums<2 * CPW, float>(sums, lane);
     constexpr int STEP = 32 / (2 * CPW);
@@ -195,22 +216,26 @@ __device__ __noinline__ int cut_qrcp_reg(Team tm, const double* A, int lda, int 
 #pragma unroll
     for (int u = 0; u < CPW; ++u) {
       const int c = warp + u * nw;
-      const float w = tau * __shfl_sync(0xffffffffu, mine, u * STEP);
+      const float w = -tau * __shfl_sync(0xffffffffu, mine, u * STEP);
       const float s = __shfl_sync(0xffffffffu, mine, (CPW + u) * STEP);
+      const uint64_t w2 = f2_pack(w, w);
+#pragma unroll
+      for (int t = 0; t < H; ++t) a[u][t] = f2_fma(w2, v[t], a[u][t]);
       float top = 0.f;
 #pragma unroll
-      for (int t = 0; t < RPL; ++t) {
-        a[u][t] -= w * v[t];
-        if (lane + 32 * t == j) top = a[u][t];
-      }
+      for (int t = 0; t < H; ++t)
+        if (t == jt) {   // the same for every thread
+          top = jh ? f2_hi(a[u][t]) : f2_lo(a[u][t]);
+          if (lane == jl) a[u][t] = jh ? f2_pack(f2_lo(a[u][t]), 0.f) : f2_pack(0.f, f2_hi(a[u][t]));
+        }
       const bool on = !((taken >> u) & 1u) && c != p;
-      if (lane == (j & 31)) {
+      if (lane == jl) {
         if (c < m) L[(size_t)j * ldl + c] = on ? top : (c == p ? alpha : 0.f);
         if (on) best = max(best, cut_key(s - top * top, c));
       }
       if (c == p) taken |= 1u << u;
     }
-    if (lane == (j & 31)) keys[warp] = best;
+    if (lane == jl) keys[warp] = best;
   }
   tm.sync();
   return j;
@@ -450,6 +475,99 @@ __device__ __noinline__ void cut_jacobi(Team tm, R* L, int ldl, int m, int r, in
   }
 }
 
+// The FP32 version, four rows per load and two per instruction: columns padded with zeros to a multiple
+// of 32 rows (rows32), ld cut_ld32.  What bounds it is instructions (18 per 4 rows of a pair against
+// ~80 one by one) and the latency of a step (~350 cycles); N4 loads per lane and column stay in
+// registers, N4 = 0 reads them twice.
+template <int N4>
+__device__ __noinline__ void cut_jacobi32(Team tm, float* L, int ldl, int rows32, int r, int g, int* flag) {
+  constexpr int N = N4 > 0 ? N4 : 1;
+  const int ne = r + (r & 1), half = ne / 2, mm = ne - 1;
+  const int ngroups = tm.nt / g, n4 = rows32 / 4;
+  const int grp = tm.tid / g, gl = tm.tid % g;
+  for (int sweep = 0; sweep < 30; ++sweep) {
+    if (tm.tid == 0) *flag = 0;
+    tm.sync();
+    bool more = false;
+    for (int k = 0; k < mm; ++k) {
+      for (int i0 = 0; i0 < half; i0 += ngroups) {
+        const int i = i0 + grp;
+        int p = k + i, q = k - i;   // round-robin pair i of step k (team_rr_pair; their order does not matter)
+        p = p >= mm ? p - mm : p;
+        q = q < 0 ? q + mm : q;
+        if (i == 0) q = mm;
+        const bool active = i < half && p < r && q < r;
+        ulonglong2* ap = reinterpret_cast<ulonglong2*>(L + (size_t)(active ? p : 0) * ldl);
+        ulonglong2* aq = reinterpret_cast<ulonglong2*>(L + (size_t)(active ? q : 0) * ldl);
+        ulonglong2 x[N], y[N];
+        uint64_t al2 = 0ull, be2 = 0ull, ga2 = 0ull;
+        if (N4 > 0) {
+#pragma unroll
+          for (int t = 0; t < N; ++t) {
+            const bool in = active && gl + t * g < n4;
+            x[t] = in ? ap[gl + t * g] : make_ulonglong2(0ull, 0ull);
+            y[t] = in ? aq[gl + t * g] : make_ulonglong2(0ull, 0ull);
+          }
+#pragma unroll
+          for (int t = 0; t < N; ++t) {
+            al2 = f2_fma(x[t].x, x[t].x, al2);
+            be2 = f2_fma(y[t].x, y[t].x, be2);
+            ga2 = f2_fma(x[t].x, y[t].x, ga2);
+            al2 = f2_fma(x[t].y, x[t].y, al2);
+            be2 = f2_fma(y[t].y, y[t].y, be2);
+            ga2 = f2_fma(x[t].y, y[t].y, ga2);
+          }
+        } else if (active) {
+#pragma unroll 4
+          for (int t = gl; t < n4; t += g) {
+            const ulonglong2 u = ap[t], v = aq[t];
+            al2 = f2_fma(u.x, u.x, al2);
+            be2 = f2_fma(v.x, v.x, be2);
+            ga2 = f2_fma(u.x, v.x, ga2);
+            al2 = f2_fma(u.y, u.y, al2);
+            be2 = f2_fma(v.y, v.y, be2);
+            ga2 = f2_fma(u.y, v.y, ga2);
+          }
+        }
+        float al = f2_lo(al2) + f2_hi(al2), be = f2_lo(be2) + f2_hi(be2), ga = f2_lo(ga2) + f2_hi(ga2);
+        for (int o = g >> 1; o > 0; o >>= 1) {
+          al += __shfl_xor_sync(0xffffffffu, al, o);
+          be += __shfl_xor_sync(0xffffffffu, be, o);
+          ga += __shfl_xor_sync(0xffffffffu, ga, o);
+        }
+        const float gg = ga * ga, ab = al * be;
+        if (active && gg > CutTol<float>::rot2() * ab) {
+          more |= gg > CutTol<float>::done2() * ab;
+          float c, s;
+          cut_rotation(al, be, ga, c, s);
+          const uint64_t c2 = f2_pack(c, c), s2 = f2_pack(s, s), m2 = f2_pack(-s, -s);
+          if (N4 > 0) {
+#pragma unroll
+            for (int t = 0; t < N; ++t)
+              if (gl + t * g < n4) {
+                ap[gl + t * g] = make_ulonglong2(f2_fma(c2, x[t].x, f2_mul(m2, y[t].x)), f2_fma(c2, x[t].y, f2_mul(m2, y[t].y)));
+                aq[gl + t * g] = make_ulonglong2(f2_fma(c2, y[t].x, f2_mul(s2, x[t].x)), f2_fma(c2, y[t].y, f2_mul(s2, x[t].y)));
+              }
+          } else {
+#pragma unroll 4
+            for (int t = gl; t < n4; t += g) {
+              const ulonglong2 u = ap[t], v = aq[t];
+              ap[t] = make_ulonglong2(f2_fma(c2, u.x, f2_mul(m2, v.x)), f2_fma(c2, u.y, f2_mul(m2, v.y)));
+              aq[t] = make_ulonglong2(f2_fma(c2, v.x, f2_mul(s2, u.x)), f2_fma(c2, v.y, f2_mul(s2, u.y)));
+            }
+          }
+        }
+      }
+      tm.sync();
+    }
+    if (more) *flag = 1;
+    tm.sync();
+    const int any = *flag;
+    tm.sync();
+    if (!any) break;
+  }
+}
+
 // Norms of the r columns and their descending order.
 template <typename R>
 __device__ __forceinline__ void cut_order(const Team& tm, const R* L, int ldl, int m, int r, R* sg, int* ord) {
@@ -570,6 +688,12 @@ static __device__ __noinline__ void cut_orthonormalise(Team tm, const double* V,
 // Leading dimension of the columns that cut_jacobi turns: = lanes per pair mod 32 at full rank, which
 // puts the lane groups of consecutive pairs on different banks.
 __host__ __device__ __forceinline__ int cut_ldl(int nt, int m) { return bank_ld32(m, team_svd_group(nt, m, m)); }
+// The same for four-row loads: eight lanes' 128 bytes on different banks (a multiple of 4; below
+// 2 cut_ldl, so that the columns fit the FP64 ones' place).
+__host__ __device__ __forceinline__ int cut_ld32(int nt, int m) {
+  const int g = team_svd_group(nt, m, m);
+  return (m + 31) / 32 * 32 + (g < 8 ? 4 * g : 0);
+}
 
 // Scratch of a cut.  Shared memory takes the small arrays, then the FP32 columns and the vectors.
 struct CutBuf {
@@ -626,7 +750,7 @@ struct CutBuf {
 __device__ __forceinline__ int cut_fp32(const Team& tm, const double* A, int lda, int n, int m, int k, int expo, float* A_g,
                                         float* L_g, float* Ls, int cap, CutBuf& b, int* slots, float** L_out, int* ldl_out) {
   const int q = n < m ? n : m, nw = tm.nt >> 5;
-  const int ldl = cut_ldl(tm.nt, m);
+  const int ldl = cut_ld32(tm.nt, m);
   const int cols = cap / ldl < q ? cap / ldl : q;
   const int cpw = (m + nw - 1) / nw;
   float* L = cols > k ? Ls : L_g;
@@ -654,11 +778,15 @@ __device__ __forceinline__ int cut_fp32(const Team& tm, const double* A, int lda
   *L_out = L;
   *ldl_out = ldl;
   if (r <= k) return r;
-  const int g = team_svd_group(tm.nt, m, r), rows = (m + g - 1) / g;
-  if (rows <= 4) cut_jacobi<float, 4>(tm, L, ldl, m, r, g, slots);
-  else if (rows <= 8) cut_jacobi<float, 8>(tm, L, ldl, m, r, g, slots);
-  else if (rows <= 16) cut_jacobi<float, 16>(tm, L, ldl, m, r, g, slots);
-  else cut_jacobi<float, 0>(tm, L, ldl, m, r, g, slots);
+  const int rows32 = (m + 31) & ~31, pad = rows32 - m;
+  for (int w = tm.tid; w < r * pad; w += tm.nt) L[(size_t)(w / pad) * ldl + m + w % pad] = 0.f;
+  tm.sync();
+  const int g = team_svd_group(tm.nt, rows32 / 4, r), n4 = (rows32 / 4 + g - 1) / g;
+  if (n4 <= 1) cut_jacobi32<1>(tm, L, ldl, rows32, r, g, slots);
+  else if (n4 <= 2) cut_jacobi32<2>(tm, L, ldl, rows32, r, g, slots);
+  else if (n4 <= 4) cut_jacobi32<4>(tm, L, ldl, rows32, r, g, slots);
+  else if (n4 <= 8 && tm.nt == 512) cut_jacobi32<8>(tm, L, ldl, rows32, r, g, slots);
+  else cut_jacobi32<0>(tm, L, ldl, rows32, r, g, slots);
   cut_order<float>(tm, L, ldl, m, r, b.sg, b.ord);
   return r;
 }
@@ -777,16 +905,85 @@ static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, 
   return ok;
 }
 
-// Cut of rank <= most (nothing to truncate): X = M (n columns of length m, column-major, ld m;
-// destroyed); U (m x r) into An (row-major), the carry R (r x n) into Cn; Qs: most x m scratch, vr:
-// 4 most, all FP64.  Returns r, or -1 when more than `most` pivots lie above the cutoff.  *rest: the
-// largest squared column norm left out over the largest of all.
+// Householder QR with column pivoting of the m x n matrix X (row-major, ld n; destroyed), m <= 64 or so:
+// a thread per column, so that every FP64 instruction works on 32 columns (a column per warp leaves
+// most lanes idle on the few rows of a cut that does not truncate).  Two barriers per step: pivot;
+// reflector (formed by one warp).  Stop and vr as cut_qrcp, the reflector's tail in column piv_j; nrm:
+// n, keys: nw.
+static __device__ __noinline__ int cut_qrcp_cols(Team tm, double* X, int m, int n, double abs2, int most, double* vr,
+                                                 double* nrm, unsigned char* taken, unsigned* keys, double& left) {
+  const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5, q = m < n ? m : n;
+  unsigned best = 0u;
+  for (int c = tm.tid; c < n; c += tm.nt) {
+    double s = 0.0;
+    for (int i = 0; i < m; ++i) s += X[(size_t)i * n + c] * X[(size_t)i * n + c];
+    nrm[c] = s;
+    taken[c] = 0;
+    best = max(best, cut_key(s, c));
+  }
+  double d02 = 0.0;
+  int j = 0;
+  left = 0.0;
+  for (; j < q; ++j) {
+    best = __reduce_max_sync(0xffffffffu, best);
+    if (lane == 0) keys[warp] = best;
+    tm.sync();
+    const unsigned key = cut_best_key(keys, nw, lane);
+    if (key == 0u) {
+      left = 0.0;
+      break;
+    }
+    const int p = (int)(kCutColMask - (key & kCutColMask));
+    const double d2 = nrm[p];
+    if (j == 0) d02 = d2;
+    left = d02 > 0.0 ? d2 / d02 : 0.0;
+    if (!(d2 > 0.0) || d2 <= abs2 * d02 || j >= most) break;
+    if (warp == 0) {
+      const double x0 = X[(size_t)j * n + p], r = sqrt(d2);
+      const double alpha = x0 >= 0.0 ? -r : r;
+      const double tau = 1.0 / (d2 + fabs(x0) * r);
+      if (lane == 0) {
+        vr[4 * j] = x0 - alpha;
+        vr[4 * j + 1] = tau;
+        vr[4 * j + 2] = alpha;
+        vr[4 * j + 3] = double(p);
+        taken[p] = 1;
+      }
+    }
+    tm.sync();
+    const double v0 = vr[4 * j], tau = vr[4 * j + 1];
+    best = 0u;
+    for (int c = tm.tid; c < n; c += tm.nt) {
+      if (taken[c]) continue;
+      const double top = X[(size_t)j * n + c];
+      double w = v0 * top;
+      for (int i = j + 1; i < m; ++i) w += X[(size_t)i * n + p] * X[(size_t)i * n + c];
+      w *= tau;
+      double s = 0.0;
+      for (int i = j + 1; i < m; ++i) {
+        const double x = X[(size_t)i * n + c] - w * X[(size_t)i * n + p];
+        X[(size_t)i * n + c] = x;
+        s += x * x;
+      }
+      X[(size_t)j * n + c] = top - w * v0;
+      nrm[c] = s;
+      best = max(best, cut_key(s, c));
+    }
+    __syncwarp();
+  }
+  tm.sync();
+  return j;
+}
+
+// Cut of rank <= most (nothing to truncate): X = M (m x n, row-major; destroyed); U (m x r) into An
+// (row-major), the carry R (r x n) into Cn; Qs: most x m scratch, vr: 4 most, nrm: n, all FP64.  Returns
+// r, or -1 when more than `most` pivots lie above the cutoff.  *rest: the largest squared column norm
+// left out over the largest of all.
 static __device__ __noinline__ int cut_rank(Team tm, double* X, int m, int n, int most, double cutoff, double* An, double* Cn,
-                                            double* Qs, double* vr, CutBuf& b, double* s0, double* rest) {
+                                            double* Qs, double* vr, double* nrm, CutBuf& b, double* s0, double* rest) {
   double left;
   const int q = m < n ? m : n;
-  const int r = cut_qrcp<double>(tm, X, m, m, n, 0, 0.0, cutoff * cutoff, most < q ? most : q, nullptr, 0, vr, b.taken,
-                                 b.keys, left);
+  const int r = cut_qrcp_cols(tm, X, m, n, cutoff * cutoff, most < q ? most : q, vr, nrm, b.taken, b.keys, left);
   if (r == 0 || (r < q && left > cutoff * cutoff)) return -1;
   const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
   for (int kk = warp; kk < r; kk += nw) {   // Q e_kk = H_0 ... H_kk e_kk, a warp per column
@@ -794,18 +991,18 @@ static __device__ __noinline__ int cut_rank(Team tm, double* X, int m, int n, in
     for (int i = lane; i < m; i += 32) x[i] = i == kk ? 1.0 : 0.0;
     for (int j = kk; j >= 0; --j) {   // a lane's rows are its own: no exchange but the dot product
       const double v0 = vr[4 * j], tau = vr[4 * j + 1];
-      const double* v = X + (size_t)(int)vr[4 * j + 3] * m;
+      const double* v = X + (int)vr[4 * j + 3];
       double w = 0.0;
       for (int i = lane; i < m; i += 32)
-        if (i >= j) w += (i == j ? v0 : v[i]) * x[i];
+        if (i >= j) w += (i == j ? v0 : v[(size_t)i * n]) * x[i];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
       w *= tau;
       for (int i = lane; i < m; i += 32)
-        if (i >= j) x[i] -= w * (i == j ? v0 : v[i]);
+        if (i >= j) x[i] -= w * (i == j ? v0 : v[(size_t)i * n]);
     }
   }
-  for (int w = tm.tid; w < r * n; w += tm.nt) Cn[w] = X[(size_t)(w % n) * m + w / n];
+  for (int w = tm.tid; w < r * n; w += tm.nt) Cn[w] = X[w];
   tm.sync();
   for (int w = tm.tid; w < r * r; w += tm.nt) {   // pivot columns: alpha on the diagonal, zero below it
     const int j = w / r, i = w % r;
@@ -837,7 +1034,7 @@ static __device__ __noinline__ int cut_full(Team tm, const double* A, int lda, d
   if (r > 1) {
     const int g = team_svd_group(tm.nt, m, r);
     if ((m + g - 1) / g <= 8) cut_jacobi<double, 8>(tm, L, ldl, m, r, g, slots);
-    else cut_jacobi<double, 0>(tm, L, ldl, m, r, g, slots);
+      else cut_jacobi<double, 0>(tm, L, ldl, m, r, g, slots);
   }
   cut_order<double>(tm, L, ldl, m, r, sv, ord);
   double* srt = sv + q;

@@ -122,7 +122,7 @@ static __device__ __noinline__ int cut(Team tm, const FinalArgs& fa, const doubl
   }
   double* Q = work + fa.w_Q;
   double* Rg = work + fa.w_R;
-  const int64_t l_col = 4 * (int64_t)cut_ldl(tm.nt, m);   // bytes of an FP32 column
+  const int64_t l_col = 4 * (int64_t)cut_ld32(tm.nt, m);   // bytes of an FP32 column
   int k = -1, r32 = 0;
   double rest = 0.0;   // discarded fraction
   if (q > cm && ex > -400 && ex < 400) {
@@ -170,20 +170,21 @@ static __device__ __noinline__ int cut(Team tm, const FinalArgs& fa, const doubl
     }
   }
   if (k < 0 && r32 <= cm) {
-    const int64_t need_v = 8 * (4 * (int64_t)kk), need_q = 8 * (int64_t)kk * m, need_x = 8 * (int64_t)m * n;
+    const int64_t need_v = 8 * (4 * (int64_t)kk + n), need_q = 8 * (int64_t)kk * m, need_x = 8 * (int64_t)m * n;
     if (need_v + need_q <= wleft) {
       const bool xs = need_v + need_q + need_x <= pool;
       unsigned char* base = xs ? sp : wp;
       double* vr = reinterpret_cast<double*>(base);
-      double* Qs = vr + 4 * kk;
+      double* nrm = vr + 4 * kk;
+      double* Qs = nrm + n;
       double* X = xs ? Qs + (size_t)kk * m : Q;
-      for (int w = tm.tid; w < m * n; w += tm.nt) X[w] = MT[(size_t)(w % m) * ldm + w / m];
+      for (int w = tm.tid; w < m * n; w += tm.nt) X[w] = MT[(size_t)(w / n) * ldm + w % n];
       tm.sync();
-      k = cut_rank(tm, X, m, n, kk, fa.svd_cutoff, An, Cn, Qs, vr, cb, s0, &rest);
+      k = cut_rank(tm, X, m, n, kk, fa.svd_cutoff, An, Cn, Qs, vr, nrm, cb, s0, &rest);
     }
   }
   if (k < 0) {
-    const int64_t need_l = 2 * l_col * q, need_x = 8 * (int64_t)m * n;
+    const int64_t need_l = 8 * (int64_t)cut_ldl(tm.nt, m) * q, need_x = 8 * (int64_t)m * n;
     const bool ls = need_l <= pool, xs = ls && need_l + need_x <= pool;
     double* L = ls ? reinterpret_cast<double*>(sp) : Rg;
     double* X = xs ? reinterpret_cast<double*>(sp + need_l) : Q;
