@@ -241,20 +241,18 @@ __device__ __noinline__ int cut_qrcp_reg(Team tm, const double* A, int lda, int 
   return j;
 }
 
-// The same factorisation of A (n x m, lda; destroyed) in memory, FP32 or FP64: four columns at a time,
-// one barrier per step (every warp forms the reflector from the pivot column, which is only read).
-// vr != null: vr[4 j ..] = (v_0, 2 / v.v, R[j][piv_j], piv_j) of reflector j, whose tail stays in
-// column piv_j of A.  left: the largest remaining norm^2 over the first.  nr: 2 m values, keys: 2 nw.
-template <typename R>
-__device__ __noinline__ int cut_qrcp(Team tm, R* A, int lda, int n, int m, int k, R rel2, R abs2, int most, R* L, int ldl,
-                                     R* vr, unsigned char* taken, unsigned* keys, R& left) {
+// The same factorisation with the copy A (n x m, ld n; destroyed) in memory, for cuts whose copy the
+// registers do not hold: four columns at a time, one barrier per step (every warp forms the reflector
+// from the pivot column, which is only read).  keys: 2 nw.
+static __device__ __noinline__ int cut_qrcp_mem(Team tm, float* A, int n, int m, int k, float rel2, float abs2, int most,
+                                                float* L, int ldl, unsigned char* taken, unsigned* keys) {
   constexpr int CB = 4;
   const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
   {
     unsigned key = 0u;
     for (int c = warp; c < m; c += nw) {
-      const R* a = A + (size_t)c * lda;
-      R s = R(0);
+      const float* a = A + (size_t)c * n;
+      float s = 0.f;
       for (int i = lane; i < n; i += 32) s += a[i] * a[i];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -264,68 +262,57 @@ __device__ __noinline__ int cut_qrcp(Team tm, R* A, int lda, int n, int m, int k
     if (lane == 0) keys[warp] = key;
   }
   const int q = n < m ? n : m;
-  R d02 = R(0), dk2 = R(0);
+  float d02 = 0.f, dk2 = 0.f;
   int j = 0;
-  left = R(0);
-  for (; j < q; ++j) {
+  for (; j < q && j < most; ++j) {
     tm.sync();
     const unsigned key = cut_best_key(keys + (j & 1) * nw, nw, lane);
-    if (key == 0u) {
-      left = R(0);
-      break;
-    }
+    if (key == 0u) break;
     const int p = (int)(kCutColMask - (key & kCutColMask));
-    const R* ap = A + (size_t)p * lda;
-    R d2 = R(0);
+    const float* ap = A + (size_t)p * n;
+    float d2 = 0.f;
     for (int i = j + lane; i < n; i += 32) d2 += ap[i] * ap[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) d2 += __shfl_xor_sync(0xffffffffu, d2, o);
     if (j == 0) d02 = d2;
     if (j < k) dk2 = d2;
-    left = d02 > R(0) ? d2 / d02 : R(0);
-    if (!(d2 > R(0)) || d2 <= rel2 * dk2 || d2 <= abs2 * d02 || j >= most) break;
-    const R x0 = ap[j], nrm = sqrt(d2);
-    const R alpha = x0 >= R(0) ? -nrm : nrm;
-    const R v0 = x0 - alpha, tau = R(1) / (d2 + fabs(x0) * nrm);
-    if (vr && tm.tid == 0) {
-      vr[4 * j] = v0;
-      vr[4 * j + 1] = tau;
-      vr[4 * j + 2] = alpha;
-      vr[4 * j + 3] = R(p);
-    }
+    if (!(d2 > 0.f) || d2 <= rel2 * dk2 || d2 <= abs2 * d02) break;
+    const float x0 = ap[j], nrm = sqrtf(d2);
+    const float alpha = x0 >= 0.f ? -nrm : nrm;
+    const float v0 = x0 - alpha, tau = 1.f / (d2 + fabsf(x0) * nrm);
     unsigned best = 0u;
     for (int c0 = warp * CB; c0 < m; c0 += nw * CB) {
-      R dots[CB], top[CB];
-      R* ac[CB];
+      float dots[CB], top[CB];
+      float* ac[CB];
       unsigned on = 0u;
 #pragma unroll
       for (int u = 0; u < CB; ++u) {
         const int c = c0 + u;
         const bool o = c < m && c != p && !taken[c < m ? c : 0];
         on |= (unsigned)o << u;
-        ac[u] = A + (size_t)(o ? c : p) * lda;
-        dots[u] = R(0);
+        ac[u] = A + (size_t)(o ? c : p) * n;
+        dots[u] = 0.f;
         top[u] = ac[u][j];
       }
       if (on)
 #pragma unroll 2
         for (int i = j + 1 + lane; i < n; i += 32) {
-          const R v = ap[i];
+          const float v = ap[i];
 #pragma unroll
           for (int u = 0; u < CB; ++u) dots[u] += v * ac[u][i];
         }
-      const R dot = cut_warp_sums<CB, R>(dots, lane);
-      R w[CB], ss[CB];
+      const float dot = cut_warp_sums<CB, float>(dots, lane);
+      float w[CB], ss[CB];
 #pragma unroll
       for (int u = 0; u < CB; ++u) {
         w[u] = tau * (__shfl_sync(0xffffffffu, dot, u * (32 / CB)) + v0 * top[u]);
-        ss[u] = R(0);
+        ss[u] = 0.f;
       }
       if (on)
 #pragma unroll 2
         for (int i = j + 1 + lane; i < n; i += 32) {
-          const R v = ap[i];
-          R x[CB];
+          const float v = ap[i];
+          float x[CB];
 #pragma unroll
           for (int u = 0; u < CB; ++u) {
             x[u] = ac[u][i] - w[u] * v;
@@ -336,15 +323,15 @@ __device__ __noinline__ int cut_qrcp(Team tm, R* A, int lda, int n, int m, int k
             if ((on >> u) & 1u) ac[u][i] = x[u];
         }
       // the norms below row j summed afresh: the stop is decided on them
-      const R below = cut_warp_sums<CB, R>(ss, lane);
+      const float below = cut_warp_sums<CB, float>(ss, lane);
 #pragma unroll
       for (int u = 0; u < CB; ++u) {
         const int c = c0 + u;
-        const R s = __shfl_sync(0xffffffffu, below, u * (32 / CB));
+        const float s = __shfl_sync(0xffffffffu, below, u * (32 / CB));
         const bool o = (on >> u) & 1u;
         if (lane == 0 && c < m) {
-          const R x = top[u] - w[u] * v0;   // R[j][c]
-          if (L) L[(size_t)j * ldl + c] = o ? x : (c == p ? alpha : R(0));
+          const float x = top[u] - w[u] * v0;   // R[j][c]
+          L[(size_t)j * ldl + c] = o ? x : (c == p ? alpha : 0.f);
           if (o) ac[u][j] = x;
           if (c == p) taken[c] = 1;
         }
@@ -357,125 +344,93 @@ __device__ __noinline__ int cut_qrcp(Team tm, R* A, int lda, int n, int m, int k
   return j;
 }
 
-template <typename R>
-struct CutTol;
-template <>
-struct CutTol<float> {   // rotate above ~FP32 rounding; done when a sweep saw nothing above 3e-4
-  static __device__ __forceinline__ float rot2() { return 1e-12f; }
-  static __device__ __forceinline__ float done2() { return 1e-7f; }
-};
-template <>
-struct CutTol<double> {  // as TeamTol<double>; a sweep that saw nothing above 1e-8 leaves 1e-16
-  static __device__ __forceinline__ double rot2() { return 1e-30; }
-  static __device__ __forceinline__ double done2() { return 1e-16; }
-};
+// FP32 Jacobi: rotates above ~FP32 rounding; done when a sweep saw no |cos| above 3e-4 (which leaves
+// ~1e-7: the convergence is quadratic).
+constexpr float kCutRot2 = 1e-12f, kCutDone2 = 1e-7f;
 __device__ __forceinline__ void cut_rotation(float al, float be, float ga, float& c, float& s) {
   const float zeta = __fdividef(be - al, 2.f * ga), w = 1.f + zeta * zeta;
   const float t = copysignf(__fdividef(1.f, fabsf(zeta) + w * rsqrtf(w)), zeta);
   c = rsqrtf(1.f + t * t);
   s = t * c;
 }
-__device__ __forceinline__ void cut_rotation(double al, double be, double ga, double& c, double& s) {
-  const double zeta = (be - al) / (2.0 * ga);
-  const double t = copysign(1.0 / (fabs(zeta) + sqrt(1.0 + zeta * zeta)), zeta);
-  c = rsqrt(1.0 + t * t);
-  s = t * c;
-}
 
-// One-sided Jacobi of the r columns (length m, ldl) of L, without V.  g lanes per pair, one barrier
-// per step; NR > 0: both columns' rows of a lane (at most NR) stay in registers between dot and
-// rotation.  The convergence is quadratic, so the sweep that sees no |cos| above the square root of
-// the tolerance is the last.
-template <typename R, int NR>
-__device__ __noinline__ void cut_jacobi(Team tm, R* L, int ldl, int m, int r, int g, int* flag) {
-  constexpr int N = NR > 0 ? NR : 1;
+// FP64 one-sided Jacobi of the r columns (length m, ldl) of L, without V.  As in the truncation cores
+// (core.cu, group_jacobi) an FP64 instruction costs the same for one lane as for 32, so the inner
+// products take few lanes per pair (at most four warps in all), the angles one lane per pair, and the
+// rotations of the pairs that rotate are spread over all threads row by row.  The convergence is
+// quadratic, so the sweep that sees no |cos| above 1e-8 is the last.  buf: 5 (r + 1) / 2 doubles, list:
+// (r + 1) / 2 ints, slots: four shared ints.
+static __device__ __noinline__ void cut_jacobi64(Team tm, double* L, int ldl, int m, int r, double* buf, int* list,
+                                                 int* slots) {
   const int ne = r + (r & 1), half = ne / 2, mm = ne - 1;
-  const int ngroups = tm.nt / g;
-  const int grp = tm.tid / g, gl = tm.tid % g;
-  for (int sweep = 0; sweep < 30; ++sweep) {
-    if (tm.tid == 0) *flag = 0;
-    tm.sync();
-    bool more = false;
+  double *al = buf, *be = al + half, *ga = be + half, *cs = ga + half, *sn = cs + half;
+  int g = 1;
+  while (g < 32 && 2 * g * half <= 128) g *= 2;
+  const int ngroups = tm.nt / g, grp = tm.tid / g, gl = tm.tid % g;
+  for (int sweep = 0; sweep < 40; ++sweep) {
+    if (tm.tid == 0) slots[0] = 0;
     for (int k = 0; k < mm; ++k) {
+      int* cnt = slots + 1 + (k & 1);
+      if (tm.tid == 0) *cnt = 0;
       for (int i0 = 0; i0 < half; i0 += ngroups) {
         const int i = i0 + grp;
-        int p = k + i, q = k - i;   // round-robin pair i of step k (team_rr_pair)
-        p = p >= mm ? p - mm : p;
-        q = q < 0 ? q + mm : q;
-        if (i == 0) q = mm;
-        if (p > q) {
-          const int t = p;
-          p = q;
-          q = t;
-        }
+        int p = 0, q = 0;
+        if (i < half) team_rr_pair(k, i, ne, p, q);
         const bool active = i < half && q < r;
-        R* ap = L + (size_t)(active ? p : 0) * ldl;
-        R* aq = L + (size_t)(active ? q : 0) * ldl;
-        R x[N], y[N];
-        R al = R(0), be = R(0), ga = R(0);
-        if (NR > 0) {
-#pragma unroll
-          for (int t = 0; t < N; ++t) {
-            const int row = gl + t * g;
-            const bool in = active && row < m;
-            x[t] = in ? ap[row] : R(0);
-            y[t] = in ? aq[row] : R(0);
-          }
-#pragma unroll
-          for (int t = 0; t < N; ++t) {
-            al += x[t] * x[t];
-            be += y[t] * y[t];
-            ga += x[t] * y[t];
-          }
-        } else if (active) {
-#pragma unroll 4
+        double x2 = 0.0, y2 = 0.0, xy = 0.0;
+        if (active) {
+          const double* ap = L + (size_t)p * ldl;
+          const double* aq = L + (size_t)q * ldl;
           for (int row = gl; row < m; row += g) {
-            const R u = ap[row], v = aq[row];
-            al += u * u;
-            be += v * v;
-            ga += u * v;
+            const double u = ap[row], v = aq[row];
+            x2 += u * u;
+            y2 += v * v;
+            xy += u * v;
           }
         }
-        for (int o = g >> 1; o > 0; o >>= 1) {
-          al += __shfl_xor_sync(0xffffffffu, al, o);
-          be += __shfl_xor_sync(0xffffffffu, be, o);
-          ga += __shfl_xor_sync(0xffffffffu, ga, o);
-        }
-        const R g2 = ga * ga, ab = al * be;
-        if (active && g2 > CutTol<R>::rot2() * ab) {
-          more |= g2 > CutTol<R>::done2() * ab;
-          R c, s;
-          cut_rotation(al, be, ga, c, s);
-          if (NR > 0) {
-#pragma unroll
-            for (int t = 0; t < N; ++t) {
-              const int row = gl + t * g;
-              if (row < m) {
-                ap[row] = c * x[t] - s * y[t];
-                aq[row] = s * x[t] + c * y[t];
-              }
-            }
-          } else {
-#pragma unroll 4
-            for (int row = gl; row < m; row += g) {
-              const R u = ap[row], v = aq[row];
-              ap[row] = c * u - s * v;
-              aq[row] = s * u + c * v;
-            }
+        if (i0 + (tm.tid & ~31) / g < half)   // a warp without a pair has nothing to add
+          for (int o = g >> 1; o > 0; o >>= 1) {
+            x2 += __shfl_xor_sync(0xffffffffu, x2, o);
+            y2 += __shfl_xor_sync(0xffffffffu, y2, o);
+            xy += __shfl_xor_sync(0xffffffffu, xy, o);
           }
+        if (gl == 0 && i < half) {
+          al[i] = x2;
+          be[i] = y2;
+          ga[i] = active ? xy : 0.0;
         }
       }
       tm.sync();
+      for (int i = tm.tid; i < half; i += tm.nt) {
+        double c, s;
+        if (jacobi_rot(al[i], be[i], ga[i], TeamTol<double>::rel(), c, s)) {
+          cs[i] = c;
+          sn[i] = s;
+          list[atomicAdd(cnt, 1)] = i;
+          if (ga[i] * ga[i] > 1e-16 * (al[i] * be[i])) slots[0] = 1;
+        }
+      }
+      tm.sync();
+      const int tasks = *cnt * m;
+      for (int t = tm.tid; t < tasks; t += tm.nt) {
+        const int i = list[t / m], row = t % m;
+        int p, q;
+        team_rr_pair(k, i, ne, p, q);
+        double* xp = L + (size_t)p * ldl + row;
+        double* xq = L + (size_t)q * ldl + row;
+        const double c = cs[i], s = sn[i], u = *xp, v = *xq;
+        *xp = c * u - s * v;
+        *xq = s * u + c * v;
+      }
+      tm.sync();
     }
-    if (more) *flag = 1;
-    tm.sync();
-    const int any = *flag;
+    const int any = slots[0];
     tm.sync();
     if (!any) break;
   }
 }
 
-// The FP32 version, four rows per load and two per instruction: columns padded with zeros to a multiple
+// FP32 one-sided Jacobi of the r columns of L, without V, four rows per load and two per instruction: columns padded with zeros to a multiple
 // of 32 rows (rows32), ld cut_ld32.  What bounds it is instructions (18 per 4 rows of a pair against
 // ~80 one by one) and the latency of a step (~350 cycles); N4 loads per lane and column stay in
 // registers, N4 = 0 reads them twice.
@@ -536,8 +491,8 @@ __device__ __noinline__ void cut_jacobi32(Team tm, float* L, int ldl, int rows32
           ga += __shfl_xor_sync(0xffffffffu, ga, o);
         }
         const float gg = ga * ga, ab = al * be;
-        if (active && gg > CutTol<float>::rot2() * ab) {
-          more |= gg > CutTol<float>::done2() * ab;
+        if (active && gg > kCutRot2 * ab) {
+          more |= gg > kCutDone2 * ab;
           float c, s;
           cut_rotation(al, be, ga, c, s);
           const uint64_t c2 = f2_pack(c, c), s2 = f2_pack(s, s), m2 = f2_pack(-s, -s);
@@ -770,8 +725,7 @@ __device__ __forceinline__ int cut_fp32(const Team& tm, const double* A, int lda
       for (int c = tm.tid >> 5; c < m; c += nw)
         for (int i = lane; i < n; i += 32) A_g[(size_t)c * n + i] = cut_f32(A[(size_t)c * lda + i], expo);
       tm.sync();
-      float left;
-      r = cut_qrcp<float>(tm, A_g, n, n, m, k, 1e-6f, 1e-12f, most, L, ldl, nullptr, b.taken, b.keys, left);
+      r = cut_qrcp_mem(tm, A_g, n, m, k, 1e-6f, 1e-12f, most, L, ldl, b.taken, b.keys);
     }
     if (r < most || most == q) break;
   }
@@ -1015,27 +969,33 @@ static __device__ __noinline__ int cut_rank(Team tm, double* X, int m, int n, in
   return r;
 }
 
-// Any cut, in FP64: pivoted QR of A (X: a copy, ld n; destroyed), Jacobi on R^T (L, ld
-// cut_ldl); sv: 2 min(m, n) singular values (unsorted, then sorted), ord: their
-// order.  Returns the number kept by the rule (0: the matrix is zero or not finite); U into An,
-// the carry into Cn; *rest: the discarded fraction.
+// Any cut, in FP64: pivoted QR of A (X: n x m scratch), Jacobi on R^T (L, ld cut_ldl); vr: 4 q doubles,
+// nrm: max(m, 5 (q + 1) / 2), list: m + q ints (q = min(m, n)); sv: 2 q singular values (unsorted, then
+// sorted), ord: their order; slots: four shared ints.  Returns the number kept by the rule (0: the
+// matrix is zero or not finite); U into An, the carry into Cn; *rest: the discarded fraction.
 static __device__ __noinline__ int cut_full(Team tm, const double* A, int lda, double* X, int m, int n, int most,
-                                            double cutoff, double rtol, double* L, double* sv, int* ord, double* An,
-                                            double* Cn, CutBuf& b, int* slots, double* s0, double* rest) {
-  const int lane = tm.tid & 31, nw = tm.nt >> 5, q = n < m ? n : m;
-  for (int c = tm.tid >> 5; c < m; c += nw)
-    for (int i = lane; i < n; i += 32) X[(size_t)c * n + i] = A[(size_t)c * lda + i];
+                                            double cutoff, double rtol, double* L, double* vr, double* nrm, int* list,
+                                            double* sv, int* ord, double* An, double* Cn, CutBuf& b, int* slots,
+                                            double* s0, double* rest) {
+  const int q = n < m ? n : m;
+  for (int w = tm.tid; w < m * n; w += tm.nt) X[w] = A[(size_t)(w % m) * lda + w / m];
   tm.sync();
   double left;
-  const int ldl = cut_ldl(tm.nt, m);
   // directions below 1e-15 of the largest are rounding of A
-  const int r = cut_qrcp<double>(tm, X, n, n, m, 0, 0.0, 1e-30, q, L, ldl, nullptr, b.taken, b.keys, left);
+  const int r = cut_qrcp_cols(tm, X, n, m, 1e-30, q, vr, nrm, b.taken, b.keys, left);
   if (r == 0) return 0;
-  if (r > 1) {
-    const int g = team_svd_group(tm.nt, m, r);
-    if ((m + g - 1) / g <= 8) cut_jacobi<double, 8>(tm, L, ldl, m, r, g, slots);
-      else cut_jacobi<double, 0>(tm, L, ldl, m, r, g, slots);
+  const int ldl = cut_ldl(tm.nt, m);
+  int* step = list;   // the step in which a column was the pivot
+  for (int c = tm.tid; c < m; c += tm.nt) step[c] = r;
+  tm.sync();
+  for (int j = tm.tid; j < r; j += tm.nt) step[(int)vr[4 * j + 3]] = j;
+  tm.sync();
+  for (int w = tm.tid; w < r * m; w += tm.nt) {
+    const int j = w / m, c = w % m;
+    L[(size_t)j * ldl + c] = j < step[c] ? X[w] : (j == step[c] ? vr[4 * j + 2] : 0.0);
   }
+  tm.sync();
+  if (r > 1) cut_jacobi64(tm, L, ldl, m, r, nrm, list + m, slots);
   cut_order<double>(tm, L, ldl, m, r, sv, ord);
   double* srt = sv + q;
   for (int i = tm.tid; i < r; i += tm.nt) srt[i] = sv[ord[i]];

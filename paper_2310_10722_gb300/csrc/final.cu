@@ -184,12 +184,24 @@ static __device__ __noinline__ int cut(Team tm, const FinalArgs& fa, const doubl
     }
   }
   if (k < 0) {
-    const int64_t need_l = 8 * (int64_t)cut_ldl(tm.nt, m) * q, need_x = 8 * (int64_t)m * n;
-    const bool ls = need_l <= pool, xs = ls && need_l + need_x <= pool;
-    double* L = ls ? reinterpret_cast<double*>(sp) : Rg;
-    double* X = xs ? reinterpret_cast<double*>(sp + need_l) : Q;
-    k = cut_full(tm, MT, ldm, X, m, n, cm, fa.svd_cutoff, fa.multiplet_rtol, L, work + fa.w_s,
-                 reinterpret_cast<int*>(work + fa.w_ord), An, Cn, cb, slots, s0, &rest);
+    const int ints = (m + q + 1) & ~1, nb = m > 5 * (q + 1) / 2 ? m : 5 * (q + 1) / 2;
+    const int64_t need_v = 8 * (4 * (int64_t)q + nb) + 4 * ints, need_l = 8 * (int64_t)cut_ldl(tm.nt, m) * q,
+                  need_x = 8 * (int64_t)m * n;
+    const bool vs = need_v <= pool;
+    if (vs || need_v <= wleft) {
+      double* vr = reinterpret_cast<double*>(vs ? sp : wp);
+      double* nrm = vr + 4 * q;
+      int* list = reinterpret_cast<int*>(nrm + nb);
+      if (vs) {
+        sp += (need_v + 15) / 16 * 16;
+        pool -= (need_v + 15) / 16 * 16;
+      }
+      const bool ls = need_l <= pool, xs = need_l + need_x <= pool;
+      double* L = ls ? reinterpret_cast<double*>(sp) : Rg;
+      double* X = xs ? reinterpret_cast<double*>(sp + need_l) : Q;
+      k = cut_full(tm, MT, ldm, X, m, n, cm, fa.svd_cutoff, fa.multiplet_rtol, L, vr, nrm, list, work + fa.w_s,
+                   reinterpret_cast<int*>(work + fa.w_ord), An, Cn, cb, slots, s0, &rest);
+    }
   }
   if (k > 0 && fa.stats && tm.tid == 0) {
     trunc[0] = fmax(trunc[0], rest);
