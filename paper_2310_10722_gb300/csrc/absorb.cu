@@ -447,13 +447,38 @@ __global__ void __launch_bounds__(256) k_gram_sym16(SweepArgs a, const GateDesc*
   }
 }
 
+// Effective dimension of a bond: its weights are sorted and zero beyond the rank that its last
+// truncation kept, and so are the columns of both its tensors there.  One warp; n = the bond's
+// dimension (<= 32).
+__device__ __forceinline__ int bond_rank(const double* lam, int n, int lane) {
+  const bool nz = lane < n && (__double_as_longlong(lam[lane]) << 1) != 0ll;
+  const unsigned mask = __ballot_sync(0xffffffffu, nz);
+  return 32 - __clz(mask);
+}
+
 // Update pass: Gamma_new[lo] = Y T+ + Z T-, Gamma_new[hi] = Y T+ - Z T-, in FP64 arithmetic
 // for both storage types (T), the result rounded to the storage type.
+//
+// What bounds it: FP64 instructions, 2 D Dn / 32 + (D + Dn) / 16 per row and one every 19 cycles of an
+// SM.  None is spent on zeros: the tensors are padded to the static bond dimensions, so the rows are
+// enumerated over the effective dimensions of the other bonds, the sums run over the rows of T that
+// are not zero and the columns that the truncation kept; the rest of the output is zero-filled.  The
+// terms left out are exact zeros and each output's sum keeps its order, so the result is the same.
+// Column q of a row belongs to lane q % LPR, so a step of LPR columns is skipped as a whole.
+// Measured (update time of a decode, padded -> effective): see update_launch.
+template <int DMAX>
+struct UpShape;   // lanes per row
+template <>
+struct UpShape<8> { static constexpr int LPR = 2; };
+template <>
+struct UpShape<16> { static constexpr int LPR = 4; };
+template <>
+struct UpShape<32> { static constexpr int LPR = 32; };
+
 template <typename T, int DMAX>
 __global__ void __launch_bounds__(256) k_update(SweepArgs a, const GateDesc* __restrict__ gates,
-                                                    const double* __restrict__ tbuf, int64_t n_jobs, int nchunk,
-                                                    int chunk_rows) {
-  constexpr int LPR = Shape<DMAX>::LPR, BPL = DMAX / LPR, RPW = 32 / LPR;
+                                                    const double* __restrict__ tbuf, int64_t n_jobs, int nchunk) {
+  constexpr int LPR = UpShape<DMAX>::LPR, BPL = DMAX / LPR, RPW = 32 / LPR;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wpb = blockDim.x >> 5;
   const int64_t job = (int64_t)blockIdx.x * wpb + warp;
@@ -468,69 +493,139 @@ __global__ void __launch_bounds__(256) k_update(SweepArgs a, const GateDesc* __r
   const bool dg = gd.diag != 0;   // diagonal gate: the blocks are lo and hi themselves
   const int D = gd.D, Dn = gd.Dn;
   const double* tsrc = tbuf + jb.gb * 4 * chi * chi + (int64_t)jb.side * 2 * chi * chi;
+  int qe = 0, je = 0;   // rows of T+ and T- that are not all zero, columns likewise
   for (int w = lane; w < DMAX * DMAX; w += 32) {
     const int q = w / DMAX, j = w % DMAX;
     const bool in = q < D && j < Dn;
-    Tp[w] = in ? tsrc[q * Dn + j] : 0.0;
-    Tm[w] = in ? tsrc[chi * chi + q * Dn + j] : 0.0;
+    const double tp = in ? tsrc[q * Dn + j] : 0.0, tm = in ? tsrc[chi * chi + q * Dn + j] : 0.0;
+    Tp[w] = tp;
+    Tm[w] = tm;
+    if (((__double_as_longlong(tp) | __double_as_longlong(tm)) << 1) != 0ll) {
+      qe = max(qe, q + 1);
+      je = max(je, j + 1);
+    }
   }
-  __syncwarp();
+  qe = __reduce_max_sync(0xffffffffu, qe);
+  je = __reduce_max_sync(0xffffffffu, je);
+  // effective dimensions and strides of the other bonds (e: 1 for the active bond)
+  const double* lamb = a.lam + (int64_t)jb.b * a.nbonds * chi;
+  int e[kMaxBonds], sin[kMaxBonds], sout[kMaxBonds];
+  int reff = 1;
+  {
+    int si = 1, so = 1;
+#pragma unroll
+    for (int k = kMaxBonds - 1; k >= 0; --k) {
+      e[k] = 1;
+      sin[k] = sout[k] = 0;
+      if (k < sd.nb) {
+        const int dk = k == sd.pos ? D : sd.dims[k];
+        sin[k] = si;
+        sout[k] = so;
+        si *= dk;
+        so *= k == sd.pos ? Dn : dk;
+        if (k != sd.pos) e[k] = bond_rank(lamb + sd.bond[k] * chi, dk, lane);
+      }
+      reff *= e[k];
+    }
+  }
+  if (qe == 0) reff = 0;
   const Pairs pg = side_pairs(sd.P, sd.mask);
   const int OI = sd.outer * sd.inner;
-  const int rows = pg.npairs * OI;
-  const int r_begin = jb.ch * chunk_rows;
-  const int r_end = min(rows, r_begin + chunk_rows);
   const int64_t SZ = (int64_t)OI * D, SZn = (int64_t)OI * Dn;
   const T* gin = reinterpret_cast<const T*>(a.gamma) + (int64_t)jb.b * a.shot_elems + sd.in_off;
   T* gout = reinterpret_cast<T*>(a.gamma) + (int64_t)jb.b * a.shot_elems + sd.out_off;
+  // the rows without effect, and every row where nothing is left: zeros
+  if (reff < OI) {
+    const int rows = pg.npairs * OI;
+    const int r_end = (int)((int64_t)(jb.ch + 1) * rows / nchunk);
+    for (int r = (int)((int64_t)jb.ch * rows / nchunk) + lane; r < r_end; r += 32) {
+      const int pr = r / OI, oi = r % OI;
+      int o = oi / sd.inner, i = oi % sd.inner;
+      const int64_t at = (int64_t)o * Dn * sd.inner + i;
+      bool in = reff > 0;
+#pragma unroll
+      for (int k = kMaxBonds - 1; k >= 0; --k)
+        if (k < sd.nb && k != sd.pos) {
+          const int dk = sd.dims[k];
+          int& src = k > sd.pos ? i : o;
+          in &= src % dk < e[k];
+          src /= dk;
+        }
+      if (!in) {
+        T* qlo = gout + pg.lo(pr) * SZn + at;
+        T* qhi = gout + pg.hi(pr) * SZn + at;
+        for (int j = 0; j < Dn; ++j) {
+          qlo[(int64_t)j * sd.inner] = T(0);
+          qhi[(int64_t)j * sd.inner] = T(0);
+        }
+      }
+    }
+  }
+  const int rows = pg.npairs * reff;
+  const int r_begin = (int)((int64_t)jb.ch * rows / nchunk), r_end = (int)((int64_t)(jb.ch + 1) * rows / nchunk);
   const int slot = lane / LPR, sub = lane % LPR, row0 = slot * LPR;
-  const int base = sub * BPL;
   for (int r0 = r_begin; r0 < r_end; r0 += RPW) {
     const int r = r0 + slot;
     const bool live = r < r_end;
-    int pr = 0, o = 0, i = 0;
+    int pr = 0, ain = 0, aout = 0;
     if (live) {
-      pr = r / OI;
-      const int oi = r % OI;
-      o = oi / sd.inner;
-      i = oi % sd.inner;
+      int t = r;
+#pragma unroll
+      for (int k = kMaxBonds - 1; k >= 0; --k)
+        if (e[k] > 1) {
+          const int d = t % e[k];
+          t /= e[k];
+          ain += d * sin[k];
+          aout += d * sout[k];
+        }
+      pr = t;
     }
     double yo[BPL], zo[BPL];
     {
-      const T* plo = gin + pg.lo(pr) * SZ + (int64_t)o * D * sd.inner + i;
-      const T* phi = gin + pg.hi(pr) * SZ + (int64_t)o * D * sd.inner + i;
+      const T* plo = gin + pg.lo(pr) * SZ + ain;
+      const T* phi = gin + pg.hi(pr) * SZ + ain;
 #pragma unroll
       for (int k = 0; k < BPL; ++k) {
-        const int q = base + k;
-        double lo = 0.0, hi = 0.0;
-        if (live && q < D) {
-          lo = double(plo[(int64_t)q * sd.inner]);
-          hi = double(phi[(int64_t)q * sd.inner]);
+        const int q = k * LPR + sub;
+        if (k * LPR < qe) {
+          double lo = 0.0, hi = 0.0;
+          if (live && q < D) {
+            lo = double(plo[(int64_t)q * sd.inner]);
+            hi = double(phi[(int64_t)q * sd.inner]);
+          }
+          yo[k] = dg ? lo : lo + hi;
+          zo[k] = dg ? hi : lo - hi;
+        } else {
+          yo[k] = zo[k] = 0.0;
         }
-        yo[k] = dg ? lo : lo + hi;
-        zo[k] = dg ? hi : lo - hi;
       }
     }
     double y[DMAX], z[DMAX];
 #pragma unroll
     for (int q = 0; q < DMAX; ++q) {
-      y[q] = __shfl_sync(0xffffffffu, yo[q % BPL], row0 + q / BPL);
-      z[q] = __shfl_sync(0xffffffffu, zo[q % BPL], row0 + q / BPL);
+      y[q] = __shfl_sync(0xffffffffu, yo[q / LPR], row0 + q % LPR);
+      z[q] = __shfl_sync(0xffffffffu, zo[q / LPR], row0 + q % LPR);
     }
-    T* qlo = gout + pg.lo(pr) * SZn + (int64_t)o * Dn * sd.inner + i;
-    T* qhi = gout + pg.hi(pr) * SZn + (int64_t)o * Dn * sd.inner + i;
+    T* qlo = gout + pg.lo(pr) * SZn + aout;
+    T* qhi = gout + pg.hi(pr) * SZn + aout;
 #pragma unroll
     for (int k = 0; k < BPL; ++k) {
-      const int j = base + k;
+      const int j = k * LPR + sub;
       double u1 = 0.0, u2 = 0.0;
+      if (k * LPR < je) {
 #pragma unroll
-      for (int q = 0; q < DMAX; ++q) {
-        u1 += y[q] * Tp[q * DMAX + j];
-        u2 += z[q] * Tm[q * DMAX + j];
-      }
-      if (live && j < Dn) {
-        qlo[(int64_t)j * sd.inner] = T(dg ? u1 : u1 + u2);
-        qhi[(int64_t)j * sd.inner] = T(dg ? u2 : u1 - u2);
+        for (int q = 0; q < DMAX; ++q)
+          if (q < qe) {
+            u1 += y[q] * Tp[q * DMAX + j];
+            u2 += z[q] * Tm[q * DMAX + j];
+          }
+        if (live && j < Dn) {
+          qlo[(int64_t)j * sd.inner] = T(dg ? u1 : u1 + u2);
+          qhi[(int64_t)j * sd.inner] = T(dg ? u2 : u1 - u2);
+        }
+      } else if (live && j < Dn) {
+        qlo[(int64_t)j * sd.inner] = T(0);
+        qhi[(int64_t)j * sd.inner] = T(0);
       }
     }
   }
@@ -564,16 +659,34 @@ static cudaError_t gram_launch(const SweepArgs& a, const GateDesc* g, int count,
   return cudaGetLastError();
 }
 
+// The update's rows are independent, so a side is split into as many jobs as fill the chip -- about
+// kUpdateFill warps per SM, 2.5 times what an SM holds, so that uneven sides level out; at least
+// kUpdateMinRows rows each, to pay for loading T --, whatever the Gram's chunks are.  Measured, rotated d9
+// chi 16, 16 shots sweep: 146.8 ms at a fill of 16, 136.1 at 32, 130.4 at 64, 128.0 at 128, 127.6 at 256;
+// rotated d9 chi 8, 1000 shots update 93.7 ms up to 128, 95.5 at 256; 64 rows instead of 128: rotated d5,
+// 37 shots 0.69 -> 0.54 ms, 32 rows the same.  With both (padded rows in chunks of 2048 -> effective rows, split to
+// fill), update time of a decode: rotated d9 chi 8, 1000 shots 105.9 -> 93.7 ms, its FP64 152 shots
+// 18.7 -> 15.8, point d5 chi 16 152 shots 16.2 -> 9.0, rotated d5 37 shots 1.82 -> 0.54; the sweep of rotated
+// d9 chi 16, 16 shots 182 -> 136 ms.
+constexpr int kUpdateFill = 128, kUpdateMinRows = 64;
+
 template <typename T, int DMAX>
-static cudaError_t update_launch(const SweepArgs& a, const GateDesc* g, int count, const double* tbuf, int nchunk,
-                                 int chunk_rows, cudaStream_t st) {
+static cudaError_t update_launch(const SweepArgs& a, const GateDesc* g, int count, const double* tbuf, int max_rows,
+                                 cudaStream_t st) {
   const int wpb = DMAX >= 32 ? 4 : 8;
-  const int64_t n_jobs = (int64_t)count * a.B * 2 * nchunk;
+  int dev = 0, nsm = 1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int64_t sides = (int64_t)count * a.B * 2;
+  const int nchunk = (int)std::max<int64_t>(1, std::min<int64_t>((max_rows + kUpdateMinRows - 1) / kUpdateMinRows,
+                                                                ((int64_t)kUpdateFill * nsm + sides - 1) / sides));
+  const int64_t n_jobs = sides * nchunk;
   const unsigned blocks = (unsigned)((n_jobs + wpb - 1) / wpb);
   const size_t smem = (size_t)wpb * 2 * DMAX * DMAX * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(k_update<T, DMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(k_update<T, DMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_update<T, DMAX><<<blocks, wpb * 32, smem, st>>>(a, g, tbuf, n_jobs, nchunk, chunk_rows);
+  k_update<T, DMAX><<<blocks, wpb * 32, smem, st>>>(a, g, tbuf, n_jobs, nchunk);
   return cudaGetLastError();
 }
 
@@ -588,15 +701,14 @@ cudaError_t launch_gram2(const SweepArgs& a, const GateDesc* g, int count, int D
 }
 
 template <typename T>
-cudaError_t launch_update2(const SweepArgs& a, const GateDesc* g, int count, int Dm, const double* tbuf, int nchunk,
-                           int chunk_rows, cudaStream_t st) {
+cudaError_t launch_update2(const SweepArgs& a, const GateDesc* g, int count, int Dm, const double* tbuf, int max_rows,
+                           cudaStream_t st) {
   switch (absorb_dmax(Dm)) {
-    case 8: return update_launch<T, 8>(a, g, count, tbuf, nchunk, chunk_rows, st);
-    case 16: return update_launch<T, 16>(a, g, count, tbuf, nchunk, chunk_rows, st);
-    default: return update_launch<T, 32>(a, g, count, tbuf, nchunk, chunk_rows, st);
+    case 8: return update_launch<T, 8>(a, g, count, tbuf, max_rows, st);
+    case 16: return update_launch<T, 16>(a, g, count, tbuf, max_rows, st);
+    default: return update_launch<T, 32>(a, g, count, tbuf, max_rows, st);
   }
 }
-
 
 // ---- Gram pass on the tensor cores (tcgen05), exact BF16 slices ------------------------------
 // G+ = Y^T Y and G- = Z^T Z of one job (gate side, shot, row chunk) as products of BF16 slices
@@ -977,9 +1089,7 @@ template cudaError_t launch_gram_tc<double>(const SweepArgs&, const GateDesc*, i
 template cudaError_t launch_gram2<float>(const SweepArgs&, const GateDesc*, int, int, double*, int, int, cudaStream_t);
 template cudaError_t launch_gram2<double>(const SweepArgs&, const GateDesc*, int, int, double*, int, int,
                                           cudaStream_t);
-template cudaError_t launch_update2<float>(const SweepArgs&, const GateDesc*, int, int, const double*, int, int,
-                                           cudaStream_t);
-template cudaError_t launch_update2<double>(const SweepArgs&, const GateDesc*, int, int, const double*, int, int,
-                                            cudaStream_t);
+template cudaError_t launch_update2<float>(const SweepArgs&, const GateDesc*, int, int, const double*, int, cudaStream_t);
+template cudaError_t launch_update2<double>(const SweepArgs&, const GateDesc*, int, int, const double*, int, cudaStream_t);
 
 }  // namespace td

@@ -204,7 +204,7 @@ cudaError_t launch_round(const SweepArgs& a0, const GateDesc* gates, const Round
   E(TD_K_CORE);
   if (e != cudaSuccess) return e;
   B(TD_K_UPDATE);
-  e = launch_update2<T>(a, g, rd.count, D, tbuf, a.gram_chunks, cr, st);
+  e = launch_update2<T>(a, g, rd.count, D, tbuf, rd.max_rows, st);
   E(TD_K_UPDATE);
   return e;
 }

@@ -207,8 +207,8 @@ template <typename T>
 cudaError_t launch_gram_tc(const SweepArgs& a, const GateDesc* g, int count, int maxD, double* gram, int nchunk,
                            int chunk_rows, cudaStream_t st);
 template <typename T>
-cudaError_t launch_update2(const SweepArgs& a, const GateDesc* g, int count, int Dm, const double* tbuf, int nchunk,
-                           int chunk_rows, cudaStream_t st);
+cudaError_t launch_update2(const SweepArgs& a, const GateDesc* g, int count, int Dm, const double* tbuf, int max_rows,
+                           cudaStream_t st);
 
 // Static scratch of the allocation-free final contraction (final.cu).
 constexpr size_t kStaticFinalScratchBytes = size_t(64) << 20;   // 64 MiB
