@@ -450,8 +450,8 @@ __device__ void final_bwd(const AdjArgs& a, int b, double* scr, double* gbar, do
 // Per-gate scratch of the core adjoint (doubles, L2 = 2 chi; CoreScr_elems in sweep.cuh is its
 // size and must follow this carving): see gate_bwd.
 struct CoreScr {
-  double *C[2], *Uq, *Vq, *Ub, *Vb, *J, *K, *In, *Th, *Tmp, *W1, *W2, *Mx[2], *Xx[2], *Lb, *wrow;
-  __device__ CoreScr(double* base, int chi, int64_t max_oi) {
+  double *C[2], *Uq, *Vq, *Ub, *Vb, *J, *K, *In, *Th, *Tmp, *W1, *W2, *Mx[2], *Xx[2], *Lb, *P1, *P2, *si;
+  __device__ CoreScr(double* base, int chi) {
     const int L2 = 2 * chi;
     double* q = base;
     auto take = [&](int64_t n) { double* r = q; q += n; return r; };
@@ -460,7 +460,7 @@ struct CoreScr {
     J = take(L2 * chi); K = take(L2 * chi); In = take(L2 * L2); Th = take(L2 * L2); Tmp = take(L2 * L2);
     W1 = take(L2 * L2); W2 = take(L2 * L2);
     Mx[0] = take(L2 * L2); Mx[1] = take(L2 * L2); Xx[0] = take(chi * L2); Xx[1] = take(chi * L2);
-    Lb = take(4 * chi); wrow = take(max_oi);
+    Lb = take(4 * chi); P1 = take(L2 * chi); P2 = take(L2 * chi); si = take(L2);
   }
   // total size: CoreScr_elems (sweep.cuh)
 };
@@ -479,6 +479,14 @@ __device__ __forceinline__ int side_rows(const SideDesc& sd, int& lo0, int& hi0,
 // Adjoint of gate g (see the file comment).  gbar[site] holds the adjoint of the gate's
 // output tensors on entry and of its input tensors on exit; lam[bond] goes back to the
 // value before the gate; lambar[bond] becomes the adjoint of that value.
+//
+// What bounds it: FP64 instructions (19 cycles of an SM each).  Whatever does not depend on a loop's
+// inner index is formed once, with the same operations: the row weights and their inverses, the sums
+// and differences of both row contractions, the parts of U-bar and V-bar off the kept spaces, 1 / s_j.
+// The values are the same bit for bit -- the adjoint of nearly equal singular values divides by their
+// difference, so a sum regrouped here moves single entries of the gradient by 1e-8 (the one FMA per
+// term that the kappa basis would allow was built and left out for that).  Measured: rotated d7 chi 8, 152
+// shots 130 -> 86 ms.
 __device__ void gate_bwd(const AdjArgs& a, int b, int g, double* scr, double* gbar, double* lambar, double* lam,
                          double* red) {
   const GateDesc& gd = a.gates[g];
@@ -496,7 +504,7 @@ __device__ void gate_bwd(const AdjArgs& a, int b, int g, double* scr, double* gb
   const double* ordd = sv + L2;
   const int rAp = rk[0], rA = rk[0] + rk[1], rBp = rk[2], rB = rk[2] + rk[3];
   const int roff[2][2] = {{0, rAp}, {0, rBp}};
-  CoreScr cs(scr + a.o_core, chi, a.max_site);
+  CoreScr cs(scr + a.o_core, chi);
   double* rsum = scr + a.o_r;
   const double p = gd.p;
   const double cpm = 0.5 * (1.0 - 2.0 * p);
@@ -506,24 +514,49 @@ __device__ void gate_bwd(const AdjArgs& a, int b, int g, double* scr, double* gb
   double* rq = scr + a.o_xbar + 2 * a.max_site;   // per-(row, column) partial sums (see prepare_reverse)
   for (int X = 0; X < 2; ++X) {
     const SideDesc& sd = gd.side[X];
-    const int OI = sd.outer * sd.inner, Dn = gd.Dn;
+    const int OI = sd.outer * sd.inner, Dn = gd.Dn, inner = sd.inner;
     const double* Gn = hist + sd.out_off;
+    const double* Gi = hist + sd.in_off;
     const double* Gnb = gbar + (int64_t)sd.site * a.max_site;
     double* xb = scr + a.o_xbar + (int64_t)X * a.max_site;
-    for (int w = threadIdx.x; w < OI * Dn; w += blockDim.x) {
+    double* wrow = scr + a.o_w + (int64_t)X * a.max_site;   // [OI] weights, [OI] their inverses
+    double* winv = wrow + OI;
+    double* xs = scr + a.o_xs;                              // [kap][row][Dn]: xl + xh, xl - xh
+    double* ys = scr + a.o_y + (int64_t)X * a.max_site;     // [kap][row][D]: gl + gh, gl - gh
+    for (int oi = threadIdx.x; oi < OI; oi += blockDim.x) {
       int dig[kMaxBonds];
+      const double wt = env_weight(sd, oi / inner, oi % inner, lam, chi, dig);
+      wrow[oi] = wt;
+      winv[oi] = wt > 0.0 ? 1.0 / wt : 0.0;
+    }
+    bsync();
+    int lo[2], hi[2];
+    const int np = side_rows(sd, lo[0], hi[0], lo[1], hi[1]);
+    const int nrows = np * OI;
+    for (int w = threadIdx.x; w < OI * Dn; w += blockDim.x) {
       const int oi = w / Dn, j = w % Dn;
-      const int o = oi / sd.inner, i = oi % sd.inner;
-      const double wt = env_weight(sd, o, i, lam, chi, dig);
-      if (j == 0) cs.wrow[oi] = wt;
-      const double winv = wt > 0.0 ? 1.0 / wt : 0.0;
+      const int o = oi / inner, i = oi % inner;
+      const double wi = winv[oi];
       double r = 0.0;
       for (int ph = 0; ph < sd.P; ++ph) {
-        const int64_t e = (((int64_t)ph * sd.outer + o) * Dn + j) * sd.inner + i;
+        const int64_t e = (((int64_t)ph * sd.outer + o) * Dn + j) * inner + i;
         r += Gnb[e] * Gn[e];
-        xb[e] = (j < k) ? Gnb[e] * winv : 0.0;
+        xb[e] = (j < k) ? Gnb[e] * wi : 0.0;
+      }
+      for (int pr = 0; pr < np; ++pr) {
+        const double xl = xb[(((int64_t)lo[pr] * sd.outer + o) * Dn + j) * inner + i];
+        const double xh = xb[(((int64_t)hi[pr] * sd.outer + o) * Dn + j) * inner + i];
+        xs[(pr * OI + oi) * Dn + j] = xl + xh;
+        xs[(nrows + pr * OI + oi) * Dn + j] = xl - xh;
       }
       rq[w] = r;
+    }
+    for (int w = threadIdx.x; w < nrows * D; w += blockDim.x) {
+      const int row = w / D, q = w % D, pr = row / OI, oi = row % OI, o = oi / inner, i = oi % inner;
+      const double gl = Gi[(((int64_t)lo[pr] * sd.outer + o) * D + q) * inner + i];
+      const double gh = Gi[(((int64_t)hi[pr] * sd.outer + o) * D + q) * inner + i];
+      ys[w] = gl + gh;
+      ys[nrows * D + w] = gl - gh;
     }
     bsync();
     for (int oi = threadIdx.x; oi < OI; oi += blockDim.x) {
@@ -533,25 +566,20 @@ __device__ void gate_bwd(const AdjArgs& a, int b, int g, double* scr, double* gb
     }
     bsync();
     env_lambar(sd, rsum, lam, lambar, chi, -1.0, red);
-    int lo[2], hi[2];
-    const int np = side_rows(sd, lo[0], hi[0], lo[1], hi[1]);
-    const double* Gi = hist + sd.in_off;
     // C[kap][q][j]: tiles of 32 outputs; warp w takes rows w, w + nw, ...; lanes take outputs
     const int NO = 2 * D * k, nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nrows = np * OI;
     for (int o0 = 0; o0 < NO; o0 += 32) {
       const int out = o0 + lane;
       double acc = 0.0;
       if (out < NO) {
         const int kap = out / (D * k), q = (out / k) % D, j = out % k;
+        const double* y = ys + kap * nrows * D + q;
+        const double* x = xs + kap * nrows * Dn + j;
+        int oi = warp;
         for (int row = warp; row < nrows; row += nw) {
-          const int pr = row / OI, oi = row % OI;
-          const int o = oi / sd.inner, i = oi % sd.inner;
-          const double gl = Gi[(((int64_t)lo[pr] * sd.outer + o) * D + q) * sd.inner + i];
-          const double gh = Gi[(((int64_t)hi[pr] * sd.outer + o) * D + q) * sd.inner + i];
-          const double xl = xb[(((int64_t)lo[pr] * sd.outer + o) * Dn + j) * sd.inner + i];
-          const double xh = xb[(((int64_t)hi[pr] * sd.outer + o) * Dn + j) * sd.inner + i];
-          acc += cs.wrow[oi] * (kap == 0 ? (gl + gh) * (xl + xh) : (gl - gh) * (xl - xh));
+          while (oi >= OI) oi -= OI;
+          acc += wrow[oi] * (y[row * D] * x[row * Dn]);
+          oi += nw;
         }
       }
       red[threadIdx.x] = acc;
@@ -564,6 +592,8 @@ __device__ void gate_bwd(const AdjArgs& a, int b, int g, double* scr, double* gb
       }
       bsync();
     }
+    // the rows of M' for the row update: weight and basis
+    for (int w = threadIdx.x; w < 2 * nrows * D; w += blockDim.x) ys[w] = wrow[(w / D) % OI] * ys[w] * kRs2;
   }
   // (c) adjoint of the core theta = R_A Lambda' R_B^T (rA x rB) from its recorded SVD
   int rr = 0;
@@ -617,6 +647,20 @@ __device__ void gate_bwd(const AdjArgs& a, int b, int g, double* scr, double* gb
     }
     cs.In[i * L2 + j] = v;
   }
+  for (int i = threadIdx.x; i < k; i += blockDim.x) cs.si[i] = 1.0 / sv[(int)ordd[i]];
+  // U-bar - Uq J, V-bar - Vq K: the parts off the kept spaces
+  for (int w = threadIdx.x; w < rA * k; w += blockDim.x) {
+    const int r = w / k, j = w % k;
+    double p1 = cs.Ub[r * chi + j];
+    for (int i = 0; i < rr; ++i) p1 -= cs.Uq[r * L2 + i] * cs.J[i * chi + j];
+    cs.P1[r * chi + j] = p1;
+  }
+  for (int w = threadIdx.x; w < rB * k; w += blockDim.x) {
+    const int c = w / k, j = w % k;
+    double p2 = cs.Vb[c * chi + j];
+    for (int i = 0; i < rr; ++i) p2 -= cs.Vq[c * L2 + i] * cs.K[i * chi + j];
+    cs.P2[c * chi + j] = p2;
+  }
   bsync();
   for (int w = threadIdx.x; w < rr * rB; w += blockDim.x) {   // Tmp = In Vq^T  (rr x rB)
     const int i = w / rB, c = w % rB;
@@ -631,11 +675,7 @@ __device__ void gate_bwd(const AdjArgs& a, int b, int g, double* scr, double* gb
     for (int i = 0; i < rr; ++i) acc += cs.Uq[r * L2 + i] * cs.Tmp[i * L2 + c];
     for (int j = 0; j < k; ++j) {
       const double sj = sv[(int)ordd[j]];
-      double p1 = cs.Ub[r * chi + j], p2 = cs.Vb[c * chi + j];
-      for (int i = 0; i < rr; ++i) {
-        p1 -= cs.Uq[r * L2 + i] * cs.J[i * chi + j];
-        p2 -= cs.Vq[c * L2 + i] * cs.K[i * chi + j];
-      }
+      const double p1 = cs.P1[r * chi + j], p2 = cs.P2[c * chi + j];
       acc += (p1 * cs.Vq[c * L2 + j] + cs.Uq[r * L2 + j] * p2) / sj;
     }
     cs.Th[r * L2 + c] = acc;
@@ -660,7 +700,7 @@ __device__ void gate_bwd(const AdjArgs& a, int b, int g, double* scr, double* gb
     const int r = w / rB, c = w % rB;
     double a1 = cs.Th[r * L2 + c], a2 = a1;
     for (int j = 0; j < k; ++j) {
-      const double isj = 1.0 / sv[(int)ordd[j]];
+      const double isj = cs.si[j];
       a1 -= cs.Ub[r * chi + j] * cs.Vq[c * L2 + j] * isj;
       a2 -= cs.Vb[c * chi + j] * cs.Uq[r * L2 + j] * isj;
     }
@@ -732,22 +772,25 @@ __device__ void gate_bwd(const AdjArgs& a, int b, int g, double* scr, double* gb
     const int np = side_rows(sd, lo[0], hi[0], lo[1], hi[1]);
     const double* Gi = hist + sd.in_off;
     const double* xb = scr + a.o_xbar + (int64_t)X * a.max_site;
+    const double* wrow = scr + a.o_w + (int64_t)X * a.max_site;
+    const double* ys = scr + a.o_y + (int64_t)X * a.max_site;
+    const int nrows = np * OI;
     double* gout = gbar + (int64_t)sd.site * a.max_site;
     const double* Mx = cs.Mx[X];
     const double* Xx = cs.Xx[X];
     for (int w = threadIdx.x; w < OI * D; w += blockDim.x) {
-      int dig[kMaxBonds];
       const int oi = w / D, q = w % D;
       const int o = oi / sd.inner, i = oi % sd.inner;
-      const double wt = env_weight(sd, o, i, lam, chi, dig);
+      const double wt = wrow[oi];
       double r = 0.0;
       for (int pr = 0; pr < np; ++pr) {
         const int64_t bl = ((int64_t)lo[pr] * sd.outer + o) * D * sd.inner + i;
         const int64_t bh = ((int64_t)hi[pr] * sd.outer + o) * D * sd.inner + i;
+        const double* yr = ys + (pr * OI + oi) * D;
+        const double* zr = ys + (nrows + pr * OI + oi) * D;
         double lp = 0.0, hp = 0.0, lm = 0.0, hm = 0.0;   // M'-bar lo/hi at columns (+, q), (-, q)
         for (int c = 0; c < D; ++c) {
-          const double gl = Gi[bl + (int64_t)c * sd.inner], gh = Gi[bh + (int64_t)c * sd.inner];
-          const double y = wt * (gl + gh) * kRs2, z = wt * (gl - gh) * kRs2;
+          const double y = yr[c], z = zr[c];
           const double mpp = Mx[c * L2 + q], mpm = Mx[c * L2 + D + q];
           const double mmp = Mx[(D + c) * L2 + q], mmm = Mx[(D + c) * L2 + D + q];
           lp += y * mpp + z * mmp;

@@ -902,7 +902,10 @@ static td_status prepare_reverse(td_network* net, int64_t B) {
   A.o_xbar = take(3 * max_site);   // two sides' X-bar, then per-(row, column) partial sums
   A.o_r = take(max_site);
   A.o_lambar = take((int64_t)P.n_bonds * chi);
-  A.o_core = take(td::CoreScr_elems(chi, max_site));
+  A.o_xs = take(max_site);         // one side's X-bar in the kappa basis
+  A.o_y = take(2 * max_site);      // two sides' input rows in the kappa basis
+  A.o_w = take(2 * max_site);      // two sides' row weights and their inverses
+  A.o_core = take(td::CoreScr_elems(chi));
   const int64_t mF = 2LL * Dm * Dm * Dm * Dm, mT1 = (int64_t)Dm * 2 * Dm * cmx * cm, mMN = (int64_t)m_max * n_max;
   A.fo_F = take(mF); A.fo_Fb = take(mF);
   A.fo_T1 = take(mT1); A.fo_T1b = take(mT1);

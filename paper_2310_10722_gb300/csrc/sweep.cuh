@@ -73,8 +73,8 @@ struct FinalArgs {
   int64_t w_Q, w_R;          // scratch of the cuts: a copy of the matrix, the columns of its factor
   int64_t W_elems;           // size of the W region (elements)
   int32_t use_smem;          // work region in dynamic shared memory
-  int32_t cut_need;          // bytes of shared memory the FP32 half of the largest cut can use
-  int32_t cut_smem;          // bytes of it given to this launch (work region in global memory only)
+  int32_t cut_need;          // bytes of shared memory the largest cut that truncates can use
+  int32_t cut_smem;          // bytes of it given to this launch
   int32_t smem_sm, smem_block;   // shared memory of one SM, largest per block (bytes)
   int32_t threads;           // threads per block (one block per shot)
   int32_t nbonds, chi, nslots, slot;
@@ -126,7 +126,7 @@ struct AdjArgs {
   int32_t n_det, wave_first;
   double* scratch;             // [B][scr_stride]
   int64_t scr_stride;
-  int64_t o_gbar, o_xbar, o_r, o_lambar, o_core, o_fin;   // offsets in a shot's scratch
+  int64_t o_gbar, o_xbar, o_xs, o_y, o_w, o_r, o_lambar, o_core, o_fin;   // offsets in a shot's scratch
   int64_t max_site;            // elements per site slot of gbar
   int64_t fo_F, fo_Fb, fo_T1, fo_T1b, fo_M, fo_Mb, fo_C0, fo_C1, fo_A0, fo_A1, fo_Ub, fo_W, fo_J, fo_In, fo_wg,
       fo_off;                  // final-contraction scratch
@@ -139,10 +139,10 @@ struct AdjArgs {
   double* Rbar;                // [B][S][8]
 };
 cudaError_t launch_adjoint(const AdjArgs& a, int threads, cudaStream_t st);
-// Scratch of the per-gate core adjoint (doubles) for bond cap chi and rows up to max_oi.
-inline int64_t CoreScr_elems(int chi, int64_t max_oi) {
+// Scratch of the per-gate core adjoint (doubles) for bond cap chi.
+inline int64_t CoreScr_elems(int chi) {
   const int64_t L2 = 2 * chi;
-  return 2 * L2 * chi + 2 * L2 * L2 + 4 * L2 * chi + 5 * L2 * L2 + 2 * L2 * L2 + 2 * chi * L2 + 4 * chi + max_oi;
+  return 2 * L2 * chi + 2 * L2 * L2 + 4 * L2 * chi + 5 * L2 * L2 + 2 * L2 * L2 + 2 * chi * L2 + 4 * chi + 2 * L2 * chi + L2;
 }
 
 struct FinalizeArgs {
