@@ -14,7 +14,9 @@
 // sums and FP32 singular vectors err by ~eps32 times the majority coset's weight, a relative
 // error of ~eps32 exp(margin) on the minority coset.  The cuts are those of cut.cuh, to FP64
 // accuracy on every path; the gradient pass's recorded forward takes a one-sided Jacobi SVD of
-// M^T with V accumulated (its records are M^T V and V).
+// M^T with V accumulated (its records are M^T V and V), bit for bit the same whatever the block: the
+// adjoint divides by differences of singular values, so another rounding here moves single entries of
+// the gradient by up to 1e-6.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -325,7 +327,15 @@ __global__ void __launch_bounds__(NT, MINB) k_final(FinalArgs fa) {
         const bool plain = k < 0;
         if (plain) {
           // one-sided Jacobi on the m columns of MT, V accumulated (the reverse sweep's record)
-          team_svd_onesided<R>(tm, MT, ldm, n, m, V, ldv, meta + 7, 40, true);
+          if constexpr (sizeof(R) == 8) {
+            const int half = (m + 1) / 2;
+            if (24 * half * 2 <= fa.cut_smem) {   // 5 doubles and an int per pair
+              double* buf = reinterpret_cast<double*>(smem_raw + (fa.use_smem ? fa.work_elems * sizeof(R) : 0));
+              block_svd_onesided(tm, MT, ldm, n, m, V, ldv, buf, reinterpret_cast<int*>(buf + 5 * half), meta + 2, 40);
+            } else {
+              team_svd_onesided<R>(tm, MT, ldm, n, m, V, ldv, meta + 7, 40, true);
+            }
+          }
           team_col_norms<R>(tm, MT, ldm, n, m, sv);
           team_sort_desc<R>(tm, sv, m, ord);
           if (tm.tid == 0) {
@@ -526,7 +536,7 @@ static cudaError_t final_launch(const FinalArgs& f, cudaStream_t st) {
   const int64_t wk = f.use_smem ? f.work_elems * (int64_t)sizeof(R) : 0;
   const int per_sm = std::max(1, std::min(MINB, (f.B + nsm - 1) / nsm));
   const int64_t room = std::min<int64_t>(f.smem_block, f.smem_sm / per_sm - 1024) - (int64_t)kFinalStaticSmem - wk;
-  const int64_t pool = f.rec ? 0 : std::max<int64_t>(0, std::min<int64_t>(room, f.cut_need)) / 16 * 16;
+  const int64_t pool = std::max<int64_t>(0, std::min<int64_t>(room, f.rec ? 48 * (f.rec_m + 2) / 2 : f.cut_need)) / 16 * 16;
   a.cut_smem = (int32_t)pool;
   const size_t smem = (size_t)(wk + pool);
   if (smem > 0) {
