@@ -83,7 +83,7 @@ __device__ __forceinline__ void load_gram(const Team& tm, const double* gram, in
 // four warps row by row; a pair's three sums are reduced side by side (3 instead of 6 instructions for
 // 4 lanes), or, when a block has fewer items than warps, by different warps.  The same operations in
 // the same order on every value: bit for bit the result of team_svd_onesided.  Measured (core time of
-// a decode, before -> now): rotated d9 chi 8, 1000 shots mixed 178 -> 129 ms, 152 shots FP64 66 -> 47
+// a decode, before -> with this; the angles' quotients in integers, ieee.cuh, took off another 6-11 %): rotated d9 chi 8, 1000 shots mixed 178 -> 129 ms, 152 shots FP64 66 -> 47
 // ms; d7 FP64, 48 shots 29.4 -> 18.9 ms; d5, 37 shots 10.1 -> 7.4 ms.
 struct GroupJacobi {
   double al[32], be[32], ga[32];   // squared norms and inner product of every pair of the step

@@ -22,6 +22,8 @@
 
 #include <cstdint>
 
+#include "ieee.cuh"
+
 namespace td {
 
 struct Team {
@@ -250,7 +252,8 @@ __device__ __forceinline__ bool below_zero(float a) { return a < 0.f; }
 // Rotation (c, s) of the one-sided Jacobi step for columns with squared norms al, be and
 // inner product ga; false when the pair is already orthogonal to working precision
 // (ga^2 <= tol^2 al be), or when a column is negligible (squared norm below tiny(); FP32
-// solves run on matrices scaled to a largest entry of 1).
+// solves run on matrices scaled to a largest entry of 1).  In FP64 the quotients and the root are formed
+// in integer arithmetic (ieee.cuh): 15 FP64 instructions instead of 40, the same values.
 template <typename R>
 __device__ __forceinline__ bool jacobi_rot(R al, R be, R ga, R tol, R& c, R& s) {
   if (is_zero(ga) || nonneg_le(al, TeamTol<R>::tiny()) || nonneg_le(be, TeamTol<R>::tiny()) ||
@@ -259,8 +262,8 @@ __device__ __forceinline__ bool jacobi_rot(R al, R be, R ga, R tol, R& c, R& s) 
     s = R(0);
     return false;
   }
-  const R zeta = (be - al) / (R(2) * ga);
-  const R t = (below_zero(zeta) ? R(-1) : R(1)) / (fabs(zeta) + sqrt(R(1) + zeta * zeta));
+  const R zeta = ieee_div(be - al, R(2) * ga);
+  const R t = ieee_div(below_zero(zeta) ? R(-1) : R(1), fabs(zeta) + ieee_sqrt(R(1) + zeta * zeta));
   c = rsqrt(R(1) + t * t);
   s = t * c;
   return true;
