@@ -734,10 +734,11 @@ cudaError_t launch_update2(const SweepArgs& a, const GateDesc* g, int count, int
 // What bounds it: FP64 and conversion instructions (19 cycles of an SM each), not the MMAs.  So the
 // bounds are taken on FP32 values (only their exponents are used), rows beyond the effective bond
 // dimensions -- exact zeros -- are left out before the blocks are formed, weights are computed once per
-// group instead of once per block and thread, and the first five slice sums are combined as integers.  All
-// of it is exact: the matrix is the same bit for bit.  Measured (Gram time of a decode): rotated d9 chi 8,
-// 1000 shots 118.6 -> 97.4 ms; rotated d5 FP32, 300 shots 2.92 -> 2.33 ms; the sweep of rotated d9 chi 16,
-// 16 shots 135.7 -> 128.0 ms.
+// group instead of once per block and thread, the first five slice sums are combined as integers, and FP64
+// values are cut two at a time into BF16 pairs.  All of it is exact: the matrix is the same bit for bit.
+// Measured (Gram time of a decode): rotated d9 chi 8, 1000 shots 118.6 -> 91.4 ms; rotated d5 FP32, 300 shots
+// 2.92 -> 2.23 ms; the sweep of rotated d9 chi 16, 16 shots 135.7 -> 126.4 ms.  Fetching the next block's
+// values during the MMA gave nothing (91.4 ms either way).
 // DPAD = 16 (bond dimensions 9..16): two operands (Y, Z) of 128 rows, two 128-column
 // accumulators.  DPAD = 8 (bond dimensions 4..8): one operand with Y's 64 rows above Z's.
 namespace {
@@ -799,8 +800,9 @@ __device__ __forceinline__ void tc_pair(float lo, float hi, float w1, float w2, 
 }
 
 // FP64 storage: slices of v with |v| < 2^E from its bit pattern: F = floor(|v| 2^(63-E)) < 2^63,
-// slice i = bits 62-7i .. 56-7i of F (as an exact float, with v's sign).
-__device__ __forceinline__ void tc_slices64(double v, int E, float (&t)[kTcSlices]) {
+// slice i = bits 62-7i .. 56-7i of F, with v's sign; two values as a BF16 pair.  128 + u is 0x4300 | u in
+// BF16, so subtracting 128 from the pair makes both exact without a conversion.
+__device__ __forceinline__ unsigned long long tc_fixed(double v, int E) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
   const int ev = (int)((bits >> 52) & 0x7FFull);
   unsigned long long F = 0ull;
@@ -812,11 +814,20 @@ __device__ __forceinline__ void tc_slices64(double v, int E, float (&t)[kTcSlice
     else if (sh > -64)
       F = mant >> (-sh);
   }
-  const unsigned sgn = (unsigned)(bits >> 63) << 31;
+  return F;
+}
+__device__ __forceinline__ void tc_slices64(double v0, double v1, int E, uint32_t (&t)[kTcSlices]) {
+  const unsigned long long F0 = tc_fixed(v0, E), F1 = tc_fixed(v1, E);
+  const uint32_t sgn = ((unsigned)__double2hiint(v0) >> 31 << 15) | ((unsigned)__double2hiint(v1) & 0x80000000u);
+  const __nv_bfloat162 k128 = __floats2bfloat162_rn(128.f, 128.f);
 #pragma unroll
   for (int i = 0; i < kTcSlices; ++i) {
-    const unsigned u = (unsigned)(F >> (56 - 7 * i)) & 0x7Fu;
-    t[i] = __uint_as_float(__float_as_uint(__int_as_float(0x4B000000 | (int)u) - 8388608.f) | sgn);
+    const int s = 56 - 7 * i;
+    const uint32_t u0 = (uint32_t)(F0 >> s) & 0x7Fu;
+    const uint32_t u1 = (uint32_t)(s >= 16 ? F1 >> (s - 16) : F1 << (16 - s)) & 0x7F0000u;
+    const uint32_t w = u0 | 0x43004300u | u1;
+    const __nv_bfloat162 h = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&w), k128);
+    t[i] = *reinterpret_cast<const uint32_t*>(&h) ^ sgn;
   }
 }
 }  // namespace
@@ -858,7 +869,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(SweepArgs a, const Ga
   double* lamv = wt + kTcGroupRows;                                              // [kMaxBonds][chi]
   float* lam32 = reinterpret_cast<float*>(lamv + kMaxBonds * a.chi);             // [kMaxBonds][chi]
   int* rowat = reinterpret_cast<int*>(lam32 + kMaxBonds * a.chi);                // [1024] offset of a row, pair in bit 30
-  __shared__ int nrows_s, amb_s;
+  __shared__ int amb_s;
   double* red = reinterpret_cast<double*>(smem_raw);   // end-of-job reduction (aliases the operands)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int chi = a.chi;
@@ -886,10 +897,18 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(SweepArgs a, const Ga
     if (tid < DPAD) colbits[tid] = 0u;
     if (tid == 0) amb_s = 0;
     // effective dimensions of the other bonds: rows beyond them are zero and left out
-    int e[kMaxBonds];
+    int e[kMaxBonds], str[kMaxBonds], reff = 1;
+    {
+      int si = 1;
 #pragma unroll
-    for (int k = 0; k < kMaxBonds; ++k)
-      e[k] = (k < sd.nb && k != sd.pos) ? bond_rank(lamb + sd.bond[k] * chi, sd.dims[k], lane) : 1;
+      for (int k = kMaxBonds - 1; k >= 0; --k) {
+        const bool other = k < sd.nb && k != sd.pos;
+        e[k] = other ? bond_rank(lamb + sd.bond[k] * chi, sd.dims[k], lane) : 1;
+        str[k] = other ? si : 0;
+        if (k < sd.nb) si *= k == sd.pos ? gd.D : sd.dims[k];
+        reff *= e[k];
+      }
+    }
     __syncthreads();
     const Pairs pg = side_pairs(sd.P, sd.mask);
     const int OI = sd.outer * sd.inner;
@@ -899,21 +918,36 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(SweepArgs a, const Ga
     const int64_t SZ = (int64_t)OI * D;
     const int inner = sd.inner;
     const T* gin = reinterpret_cast<const T*>(a.gamma) + (int64_t)jb.b * a.shot_elems + sd.in_off;
-    // whether row (o, i) has effect, and its FP32 weight
-    auto effective = [&](int o, int i, float& w) {
-      bool in = true;
-      w = 1.f;
+    // the rows with effect, counted: number of them below row r, and the digits, offset and weight of
+    // the t-th (the weight's factors in row_weight's order)
+    auto below = [&](int r) {
+      if (r == 0 || reff == 0) return 0;
+      if (r == rows) return pg.npairs * reff;
+      int c = r / OI * reff, rem = r % OI, m = reff, sz = OI;
+#pragma unroll
+      for (int k = 0; k < kMaxBonds; ++k)
+        if (k < sd.nb && k != sd.pos) {
+          sz /= sd.dims[k];
+          m /= e[k];
+          const int d = rem / sz;
+          rem -= d * sz;
+          c += min(d, e[k]) * m;
+          if (d >= e[k]) break;
+        }
+      return c;
+    };
+    auto row = [&](int t, auto& w, const auto* lv) {   // offset, pair in bit 30
+      int at = 0;
+      w = 1;
 #pragma unroll
       for (int k = kMaxBonds - 1; k >= 0; --k)
         if (k < sd.nb && k != sd.pos) {
-          const int dk = sd.dims[k];
-          int& src = k > sd.pos ? i : o;
-          const int d = src % dk;
-          src /= dk;
-          in &= d < e[k];
-          w *= lam32[k * chi + d];
+          const int q = t / e[k], d = t - q * e[k];
+          t = q;
+          at += d * str[k];
+          w *= lv[k * chi + d];
         }
-      return in;
+      return at | t << 30;
     };
     // 1. column bounds.  Only the exponent of a bound is used, so FP32 values within 2^-19 of the FP64
     // ones decide it unless a bound comes that close to a power of two (then, or out of FP32 range, the
@@ -923,12 +957,11 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(SweepArgs a, const Ga
       bool big = false;
 #pragma unroll
       for (int c = 0; c < DPAD; ++c) cm[c] = 0.f;
-      for (int r = r_begin + tid; r < r_end; r += kTcThreads) {
-        const int pr = r / OI, oi = r % OI, o = oi / inner, i = oi % inner;
+      for (int t = below(r_begin) + tid, t1 = below(r_end); t < t1; t += kTcThreads) {
         float w;
-        if (!effective(o, i, w)) continue;
-        const T* plo = gin + pg.lo(pr) * SZ + (int64_t)o * D * inner + i;
-        const T* phi = gin + pg.hi(pr) * SZ + (int64_t)o * D * inner + i;
+        const int ra = row(t, w, lam32), pr = ra >> 30, at = ra & 0x3FFFFFFF;
+        const T* plo = gin + pg.lo(pr) * SZ + at;
+        const T* phi = gin + pg.hi(pr) * SZ + at;
 #pragma unroll
         for (int c = 0; c < DPAD; ++c)
           if (c < D) cm[c] = fmaxf(cm[c], (tc_abs32(plo[(int64_t)c * inner], big) + tc_abs32(phi[(int64_t)c * inner], big)) * w);
@@ -985,30 +1018,15 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(SweepArgs a, const Ga
     for (int c = 0; c < DPAD; ++c) part[c] = 0.0;
     bool first = true;   // part is zero
     for (int g0 = r_begin; g0 < r_end && !failed; g0 += kTcGroupRows) {
-      // 2. the group's rows with effect and their weights (any order: their sums are exact)
-      if (tid == 0) nrows_s = 0;
-      __syncthreads();
-      const int g1 = min(r_end, g0 + kTcGroupRows);
-      for (int r0 = g0 + warp * 32; r0 < g1; r0 += kTcThreads) {
-        const int r = r0 + lane;
-        const int pr = r / OI, oi = r % OI, o = oi / inner, i = oi % inner;
-        float w32;
-        const bool in = r < g1 && effective(o, i, w32);
-        const unsigned mask = __ballot_sync(0xffffffffu, in);
-        int at = 0;
-        if (lane == 0) at = atomicAdd(&nrows_s, __popc(mask));
-        at = __shfl_sync(0xffffffffu, at, 0) + __popc(mask & ((1u << lane) - 1u));
-        if (in) {
-          wt[at] = row_weight<double>(sd, o, i, lamv, chi);
-          rowat[at] = (o * D * inner + i) | pr << 30;
-        }
+      // 2. the group's rows with effect and their weights
+      const int c0 = below(g0), nrows = below(min(r_end, g0 + kTcGroupRows)) - c0;
+      if (nrows == 0) continue;
+      for (int t = tid; t < nrows; t += kTcThreads) {
+        double w;
+        rowat[t] = row(c0 + t, w, lamv);
+        wt[t] = w;
       }
       __syncthreads();
-      const int nrows = nrows_s;
-      if (nrows == 0) {
-        __syncthreads();   // everybody has read nrows_s
-        continue;
-      }
       const int nblk = (nrows + KB - 1) / KB;
       for (int blk = 0; blk < nblk; ++blk) {
         const int rb = blk * KB;
@@ -1036,12 +1054,12 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(SweepArgs a, const Ga
             uint32_t pk[kTcSlices][4];
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-              float t0[kTcSlices], t1[kTcSlices];
+              // X x X gate: (lo + hi) w, (lo - hi) w; diagonal gate: lo w, hi w
               if constexpr (sizeof(T) == 4) {
+                float t0[kTcSlices], t1[kTcSlices];
                 float y1, y2;
                 const double w0 = w8[2 * v], w1 = w8[2 * v + 1];
                 const float w0a = (float)w0, w1a = (float)w1;
-                // X x X gate: (lo + hi) w, (lo - hi) w; diagonal gate: lo w, hi w
                 const float a0 = dg ? (pt ? 0.f : lo8[2 * v]) : lo8[2 * v];
                 const float b0 = dg ? (pt ? hi8[2 * v] : 0.f) : (pt ? -hi8[2 * v] : hi8[2 * v]);
                 const float a1 = dg ? (pt ? 0.f : lo8[2 * v + 1]) : lo8[2 * v + 1];
@@ -1050,18 +1068,19 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(SweepArgs a, const Ga
                 tc_slices32(y1 * sc, y2 * sc, t0);
                 tc_pair(a1, b1, w1a, (float)(w1 - (double)w1a), y1, y2);
                 tc_slices32(y1 * sc, y2 * sc, t1);
-              } else {
-                // X x X gate: (lo + hi) w, (lo - hi) w; diagonal gate: lo w, hi w
-                const double y0 = dg ? (pt ? hi8[2 * v] : lo8[2 * v]) : (pt ? lo8[2 * v] - hi8[2 * v] : lo8[2 * v] + hi8[2 * v]);
-                const double y1v = dg ? (pt ? hi8[2 * v + 1] : lo8[2 * v + 1])
-                                      : (pt ? lo8[2 * v + 1] - hi8[2 * v + 1] : lo8[2 * v + 1] + hi8[2 * v + 1]);
-                tc_slices64(y0 * w8[2 * v], E, t0);
-                tc_slices64(y1v * w8[2 * v + 1], E, t1);
-              }
 #pragma unroll
-              for (int i = 0; i < kTcSlices; ++i) {
-                const __nv_bfloat162 h = __floats2bfloat162_rn(t0[i], t1[i]);
-                pk[i][v] = *reinterpret_cast<const uint32_t*>(&h);
+                for (int i = 0; i < kTcSlices; ++i) {
+                  const __nv_bfloat162 h = __floats2bfloat162_rn(t0[i], t1[i]);
+                  pk[i][v] = *reinterpret_cast<const uint32_t*>(&h);
+                }
+              } else {
+                const double y0 = dg ? (pt ? hi8[2 * v] : lo8[2 * v]) : (pt ? lo8[2 * v] - hi8[2 * v] : lo8[2 * v] + hi8[2 * v]);
+                const double y1 = dg ? (pt ? hi8[2 * v + 1] : lo8[2 * v + 1])
+                                     : (pt ? lo8[2 * v + 1] - hi8[2 * v + 1] : lo8[2 * v + 1] + hi8[2 * v + 1]);
+                uint32_t t[kTcSlices];
+                tc_slices64(y0 * w8[2 * v], y1 * w8[2 * v + 1], E, t);
+#pragma unroll
+                for (int i = 0; i < kTcSlices; ++i) pk[i][v] = t[i];
               }
             }
             unsigned char* base = opnd + (NACC == 2 ? (size_t)pt * 128 * KB * 2 : 0);
