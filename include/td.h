@@ -308,8 +308,8 @@ td_status td_gen_rows_host(const td_gen* gen, const uint8_t* syn_host, int64_t B
  * block size of the final contraction's kernel (256, 512 or 1024 threads; the Jacobi lane
  * groups and the work region's layout follow it), whether that kernel's work region may sit
  * in shared memory (final_smem != 0: when it fits; 0: global memory, cached in L1, which
- * leaves room for more blocks per SM), and the rows per job of the Gram and update passes
- * (512, 1024, 2048 or 4096).  Results do not depend on the schedule beyond rounding (the
+ * leaves room for more blocks per SM), and the rows per job of the Gram pass (512, 1024, 2048 or
+ * 4096; the update splits its rows by itself).  Results do not depend on the schedule beyond rounding (the
  * Gram's partial sums and the Jacobi rotations are grouped differently).
  * td_network_set_schedule sets it; TD_ERR_INVALID for other values. */
 td_status td_network_set_schedule(td_network* net, int32_t final_threads, int32_t final_smem, int32_t chunk_rows);
