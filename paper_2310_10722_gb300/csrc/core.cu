@@ -85,6 +85,8 @@ __device__ __forceinline__ void load_gram(const Team& tm, const double* gram, in
 // the same order on every value: bit for bit the result of team_svd_onesided.  Measured (core time of
 // a decode, before -> with this; the angles' quotients in integers, ieee.cuh, took off another 6-11 %): rotated d9 chi 8, 1000 shots mixed 178 -> 129 ms, 152 shots FP64 66 -> 47
 // ms; d7 FP64, 48 shots 29.4 -> 18.9 ms; d5, 37 shots 10.1 -> 7.4 ms.
+// Not done: keeping the squared norms of columns that did not rotate (a twelfth fewer FP64 instructions):
+// 121.5 -> 120.5 ms with a full chip, but 6.8 -> 7.2 ms for d5, 37 shots, where a step is a chain.
 struct GroupJacobi {
   double al[32], be[32], ga[32];   // squared norms and inner product of every pair of the step
   double c[32], s[32];
