@@ -505,6 +505,7 @@ __global__ void __launch_bounds__(256) k_update(SweepArgs a, const GateDesc* __r
       je = max(je, j + 1);
     }
   }
+  __syncwarp();   // T+ and T- are read across lanes below; a reduction or ballot orders no memory
   qe = __reduce_max_sync(0xffffffffu, qe);
   je = __reduce_max_sync(0xffffffffu, je);
   // effective dimensions and strides of the other bonds (e: 1 for the active bond)
