@@ -136,7 +136,7 @@ static __device__ __noinline__ int cut(Team tm, const FinalArgs& fa, const doubl
       else cb.carve_vec(reinterpret_cast<double*>(wp), m, n, cm, Cn);
       unsigned char* lp = vs ? sp + vec_p : sp;
       const int64_t cap = (vs ? pool - vec_p : pool) / 4;
-      if (cut_topk(tm, MT, ldm, n, m, cm, ex, reinterpret_cast<float*>(Q), reinterpret_cast<float*>(Rg),
+      if (cut_topk(tm, MT, ldm, n, m, cm, fa.multiplet_rtol, ex, reinterpret_cast<float*>(Q), reinterpret_cast<float*>(Rg),
                    reinterpret_cast<float*>(lp), (int)cap, cb, slots, s0, &r32)) {
         k = cm;
         for (int w = tm.tid; w < m * k; w += tm.nt) An[w] = cb.V[w];
