@@ -20,13 +20,15 @@
 //          (FP32: T needs no more digits than it corrects).  Each pass gains the 5-7 digits of the
 //          FP32 basis, so two passes reach FP64 accuracy; V is re-orthonormalised by one
 //          Newton-Schulz step per pass.  FP64 work 10 n m k.
-//     It applies where FP32 resolves the cut (cut_resolved): sigma_k - sigma_{k+1} above the
-//     multiplet rule's threshold (multiplet_rtol) with room for FP32's error, and sigma_k >= 1e-5
+//     It applies where FP32 resolves the cut (cut_resolved): both rules of the truncation
+//     (svd_cutoff, multiplet_rtol) keep exactly k with room for FP32's error, and sigma_k >= 1e-5
 //     sigma_1; and it checks itself (the residual has to fall to FP64 rounding).
 //   * cut_rank (rank <= chi_mps: nothing to truncate): FP64 pivoted QR of M, stopped at the first
-//     pivot below svd_cutoff times the largest: U = Q, carry = R.  No SVD.
-//   * cut_full (steep spectra, cuts inside a multiplet): as 1 and 2 in FP64 throughout; every
-//     singular value, so the keep rule is decided on them.
+//     pivot below svd_cutoff times the largest: U = Q, carry = R.  No SVD.  A pivot is not a singular
+//     value -- it can be off by a factor of a few --, so this path is for cutoffs that only drop what is
+//     next to rounding anyway (kCutRankCutoff).
+//   * cut_full (steep spectra, cuts inside a multiplet, larger cutoffs): as 1 and 2 in FP64 throughout;
+//     every singular value, so the keep rule is decided on them.
 // Measured against numpy's SVD on 130 cuts of the tests' networks: U U^T M of cut_topk differs by
 // <= 6e-14 sigma_1 (median 2e-15).
 //
@@ -826,18 +828,19 @@ __device__ __forceinline__ int cut_fp32(const Team& tm, const double* A, int lda
 }
 
 // Whether the FP32 singular values t0 (the largest), tk (the k-th), tn (the next) decide the cut at k:
-// no multiplet is cut inside s_k - s_{k+1} <= rtol * t0.  A pivoted QR and an SVD in FP32 give
-// the values to 2e-7 t0 (numpy, largest error over 164 cuts of the tests' networks), so the rule has to hold
-// by 1e-6 t0; closer cuts are decided in FP64.
-__device__ __forceinline__ bool cut_resolved(float t0, float tk, float tn, double rtol) {
-  return tk >= 1e-5f * t0 && tk - tn > 1e-4f * tk && tk - tn > float(rtol) * t0 + 1e-6f * t0;
+// keep those above cutoff * t0, and none of a multiplet cut inside s_k - s_{k+1} <= rtol * t0.  A
+// pivoted QR and an SVD in FP32 give the values to 2e-7 t0 (numpy, largest error over 164 cuts of the tests'
+// networks), so both rules have to hold by 1e-6 t0; closer cuts are decided in FP64.
+__device__ __forceinline__ bool cut_resolved(float t0, float tk, float tn, double cutoff, double rtol) {
+  const float eps = 1e-6f * t0;
+  return tk >= 1e-5f * t0 && tk > float(cutoff) * t0 + eps && tk - tn > 1e-4f * tk && tk - tn > float(rtol) * t0 + eps;
 }
 
 // See the file comment.  2^expo: the magnitude of A's largest entry.  b.P receives the carry
 // U_k^T M, b.V the vectors; slots: two shared ints.  Returns false (nothing usable) when the cut is not
 // one for this path; *r32 is then the FP32 rank.
-static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, int n, int m, int k, double rtol,
-                                             int expo, float* A_g, float* L_g, float* Ls, int cap,
+static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, int n, int m, int k, double cutoff,
+                                             double rtol, int expo, float* A_g, float* L_g, float* Ls, int cap,
                                              CutBuf& b, int* slots, double* s0, int* r32) {
   const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
   float* L;
@@ -845,7 +848,7 @@ static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, 
   const int r = cut_fp32(tm, A, lda, n, m, k, expo, A_g, L_g, Ls, cap, b, slots, &L, &ldl);
   *r32 = r;
   if (r <= k) return false;
-  if (!cut_resolved(b.sg[b.ord[0]], b.sg[b.ord[k - 1]], b.sg[b.ord[k]], rtol)) return false;
+  if (!cut_resolved(b.sg[b.ord[0]], b.sg[b.ord[k - 1]], b.sg[b.ord[k]], cutoff, rtol)) return false;
   double *V = b.V, *V2 = b.V2;
   for (int w = tm.tid; w < m * k; w += tm.nt) {
     const int c = w / k, o = b.ord[w % k];
@@ -942,6 +945,11 @@ static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, 
   if (ok) *s0 = sqrt(b.th[0]);
   return ok;
 }
+
+// Largest svd_cutoff that may be applied to pivots in place of singular values.  The oracle with pivots
+// (chi_mps 16 and 64, five networks) is within 2e-13 of the keep rule in log p at cutoffs up to 1e-8, 1e-5 off
+// at 1e-4 and 1e-2 off at 3e-2; the line stands well below the first and above the default, 1e-12.
+constexpr double kCutRankCutoff = 1e-11;
 
 // Householder QR with column pivoting of the m x n matrix X (row-major, ld n; destroyed), m <= 64 or so:
 // a thread per column, so that every FP64 instruction works on 32 columns (a column per warp leaves

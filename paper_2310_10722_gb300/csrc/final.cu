@@ -136,8 +136,8 @@ static __device__ __noinline__ int cut(Team tm, const FinalArgs& fa, const doubl
       else cb.carve_vec(reinterpret_cast<double*>(wp), m, n, cm, Cn);
       unsigned char* lp = vs ? sp + vec_p : sp;
       const int64_t cap = (vs ? pool - vec_p : pool) / 4;
-      if (cut_topk(tm, MT, ldm, n, m, cm, fa.multiplet_rtol, ex, reinterpret_cast<float*>(Q), reinterpret_cast<float*>(Rg),
-                   reinterpret_cast<float*>(lp), (int)cap, cb, slots, s0, &r32)) {
+      if (cut_topk(tm, MT, ldm, n, m, cm, fa.svd_cutoff, fa.multiplet_rtol, ex, reinterpret_cast<float*>(Q),
+                   reinterpret_cast<float*>(Rg), reinterpret_cast<float*>(lp), (int)cap, cb, slots, s0, &r32)) {
         k = cm;
         for (int w = tm.tid; w < m * k; w += tm.nt) An[w] = cb.V[w];
         if (vs)
@@ -171,7 +171,7 @@ static __device__ __noinline__ int cut(Team tm, const FinalArgs& fa, const doubl
       }
     }
   }
-  if (k < 0 && r32 <= cm) {
+  if (k < 0 && r32 <= cm && fa.svd_cutoff <= kCutRankCutoff) {
     const int64_t need_v = 8 * (4 * (int64_t)kk + n), need_q = 8 * (int64_t)kk * m, need_x = 8 * (int64_t)m * n;
     if (need_v + need_q <= wleft) {
       const bool xs = need_v + need_q + need_x <= pool;

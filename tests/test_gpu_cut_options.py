@@ -1,9 +1,9 @@
-"""multiplet_rtol in the final contraction (csrc/cut.cuh) against the oracle's keep rule: values at which it,
-not chi_mps, decides cuts.
+"""svd_cutoff and multiplet_rtol in the final contraction (csrc/cut.cuh) against the oracle's keep rule:
+values at which they, not chi_mps, decide cuts.
 
 Tolerances are those of the parity tests (1e-6 in log p for the FP64 path, 1e-3 for the mixed ones); a cut
-that follows its built-in limits instead of the option is off by 4e-3 to 0.2 on these shots (the oracle
-with such cuts)."""
+that follows built-in limits, or pivots of a QR, instead of the option is off by 2e-3 to 0.2 on these shots
+(the oracle with such cuts)."""
 import numpy as np
 import pytest
 
@@ -13,11 +13,17 @@ from td_inputs import point_sector_3d, rotated_phenomenological, sample_shots
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
-ROT5, ROT5_HIGH, POINT4 = rotated_phenomenological(5, 4, 0.04, 0.04), rotated_phenomenological(5, 4, 0.08, 0.08), point_sector_3d(4, 0.1)
+ROT5, ROT5_HIGH = rotated_phenomenological(5, 4, 0.04, 0.04), rotated_phenomenological(5, 4, 0.08, 0.08)
+POINT4 = point_sector_3d(4, 0.1)
 CASES = {   # DEM, chi, chi_mps, svd_cutoff, multiplet_rtol, seed of the shots
     "multiplet of rotated d5": (ROT5, 8, 8, 1e-12, 1e-2, 1),
     "multiplet of point d4": (POINT4, 8, 8, 1e-12, 1e-2, 2),
     "multiplet of rotated d5, high rate": (ROT5_HIGH, 8, 4, 1e-12, 1e-3, 1),
+    "cutoff above the cap, rotated d5": (ROT5, 8, 4, 1e-2, 1e-8, 2),
+    "cutoff above the cap, point d4": (POINT4, 4, 6, 1e-2, 1e-8, 2),
+    "cutoff below the cap, rotated d5": (ROT5, 8, 16, 1e-3, 1e-8, 2),
+    "cutoff below the cap, rotated d5, high rate": (ROT5_HIGH, 8, 16, 1e-2, 1e-8, 2),
+    "cutoff below the cap, point d3": (point_sector_3d(3, 0.1), 8, 64, 3e-2, 1e-8, 2),
 }
 
 
