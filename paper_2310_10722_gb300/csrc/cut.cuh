@@ -37,18 +37,10 @@
 // exchange is an L2 round trip, and these loops are chains of them.
 #pragma once
 
+#include "cutnum.cuh"
 #include "team.cuh"
 
 namespace td {
-
-// FP32 value of x 2^-E, truncated to 24 bits, from the bit pattern (integer pipes only; below the
-// FP32 normal range: 0).
-__device__ __forceinline__ float cut_f32(double x, int E) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int e = (int)((hi >> 20) & 0x7FFu) - 1023 - E + 127;
-  if (e <= 0) return 0.0f;
-  return __uint_as_float((hi & 0x80000000u) | ((unsigned)e << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
-}
 
 // Largest biased exponent of the n x m column-major matrix A, through a shared int.
 __device__ __forceinline__ int cut_max_exponent(const Team& tm, const double* A, int lda, int n, int m, int* slot) {
@@ -889,18 +881,18 @@ static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, 
       }
     }
     tm.sync();
-    float worst = 0.f;
-    const float it0 = float(b.th[k]);
+    unsigned worst = 0u;
+    const double th0 = b.th[0];
     for (int w = tm.tid; w < m * k; w += tm.nt) {
       const int j = w / m, c = w % m;
       double s = b.C[w];
       for (int a = 0; a < k; ++a) s -= V[c * k + a] * b.S[a * k + j];
       const float e = float(s * b.th[k + j]);
       b.E[w] = e;
-      worst = fmaxf(worst, fabsf(e) * sqrtf(float(b.th[j]) * it0));
+      worst = max(worst, cut_residual(e, b.th[j], th0, expo));
     }
-    const unsigned wb = __reduce_max_sync(0xffffffffu, __float_as_uint(worst));
-    if (lane == 0) atomicMax(slots + 1, (int)wb);
+    worst = __reduce_max_sync(0xffffffffu, worst);
+    if (lane == 0) atomicMax(slots + 1, (int)worst);
     tm.sync();
     const float res = __int_as_float(slots[1]);
     // converged: the residual at FP64 rounding (or no longer falling just above it)

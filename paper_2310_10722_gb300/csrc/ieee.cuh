@@ -28,6 +28,7 @@ TD_IEEE_HD double ieee_value(uint64_t u) { return __longlong_as_double((long lon
 TD_IEEE_HD uint64_t ieee_mulhi(uint64_t a, uint64_t b) { return __umul64hi(a, b); }
 TD_IEEE_HD int64_t ieee_mulhi_s(int64_t a, int64_t b) { return __mul64hi(a, b); }
 TD_IEEE_HD float ieee_float(uint32_t u) { return __uint_as_float(u); }
+TD_IEEE_HD uint32_t ieee_float_bits(float x) { return __float_as_uint(x); }
 TD_IEEE_HD float ieee_rcp_est(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -45,6 +46,7 @@ TD_IEEE_HD double ieee_value(uint64_t u) { double x; std::memcpy(&x, &u, 8); ret
 TD_IEEE_HD uint64_t ieee_mulhi(uint64_t a, uint64_t b) { return (uint64_t)((unsigned __int128)a * b >> 64); }
 TD_IEEE_HD int64_t ieee_mulhi_s(int64_t a, int64_t b) { return (int64_t)((__int128)a * b >> 64); }
 TD_IEEE_HD float ieee_float(uint32_t u) { float x; std::memcpy(&x, &u, 4); return x; }
+TD_IEEE_HD uint32_t ieee_float_bits(float x) { uint32_t u; std::memcpy(&u, &x, 4); return u; }
 TD_IEEE_HD float ieee_rcp_est(float x) { return 1.0f / x; }
 TD_IEEE_HD float ieee_rsqrt_est(float x) { return 1.0f / std::sqrt(x); }
 #endif
