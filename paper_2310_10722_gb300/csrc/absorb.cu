@@ -463,7 +463,8 @@ __device__ __forceinline__ int bond_rank(const double* lam, int n, int lane) {
 // SM.  None is spent on zeros: the tensors are padded to the static bond dimensions, so the rows are
 // enumerated over the effective dimensions of the other bonds, the sums run over the rows of T that
 // are not zero and the columns that the truncation kept; the rest of the output is zero-filled.  The
-// terms left out are exact zeros and each output's sum keeps its order, so the result is the same.
+// terms left out are exact zeros and each output's sum keeps its order, so the result is the same for finite
+// tensors; a value that overflows is marked where it is stored (mark_non_finite).
 // Column q of a row belongs to lane q % LPR, so a step of LPR columns is skipped as a whole.
 // Measured (update time of a decode, padded -> effective): see update_launch.
 template <int DMAX>
@@ -565,6 +566,7 @@ __global__ void __launch_bounds__(256) k_update(SweepArgs a, const GateDesc* __r
   const int rows = pg.npairs * reff;
   const int r_begin = (int)((int64_t)jb.ch * rows / nchunk), r_end = (int)((int64_t)(jb.ch + 1) * rows / nchunk);
   const int slot = lane / LPR, sub = lane % LPR, row0 = slot * LPR;
+  bool over = false;   // a value that the storage type does not hold
   for (int r0 = r_begin; r0 < r_end; r0 += RPW) {
     const int r = r0 + slot;
     const bool live = r < r_end;
@@ -621,8 +623,10 @@ __global__ void __launch_bounds__(256) k_update(SweepArgs a, const GateDesc* __r
             u2 += z[q] * Tm[q * DMAX + j];
           }
         if (live && j < Dn) {
-          qlo[(int64_t)j * sd.inner] = T(dg ? u1 : u1 + u2);
-          qhi[(int64_t)j * sd.inner] = T(dg ? u2 : u1 - u2);
+          const T vlo = T(dg ? u1 : u1 + u2), vhi = T(dg ? u2 : u1 - u2);
+          qlo[(int64_t)j * sd.inner] = vlo;
+          qhi[(int64_t)j * sd.inner] = vhi;
+          over |= non_finite(vlo) || non_finite(vhi);
         }
       } else if (live && j < Dn) {
         qlo[(int64_t)j * sd.inner] = T(0);
@@ -630,6 +634,7 @@ __global__ void __launch_bounds__(256) k_update(SweepArgs a, const GateDesc* __r
       }
     }
   }
+  if (over) mark_non_finite(a, jb.b);
 }
 
 // ---- launchers -----------------------------------------------------------------------------

@@ -305,8 +305,14 @@ __global__ void k_core2(SweepArgs a, const GateDesc* __restrict__ gates, const d
   if (tm.tid < 4) {
     const int side = tm.tid / 2;
     double e = 0.0;
+    bool over = false;
     for (int blk = 2 * side; blk < 2 * side + 2; ++blk)
-      for (int j = 0; j < D; ++j) e = fmax(e, RG[blk * DD + j * D + j]);
+      for (int j = 0; j < D; ++j) {
+        const double g = RG[blk * DD + j * D + j];
+        over |= non_finite(g);
+        e = fmax(e, g);
+      }
+    if (over) mark_non_finite(a, b);
     sm.sv[tm.tid] = e > 0.0 ? a.gram_cutoff * e : -1.0;
   }
   tm.sync();
@@ -407,7 +413,10 @@ __global__ void k_core2(SweepArgs a, const GateDesc* __restrict__ gates, const d
   if (k == 0 || !(s0 > 0.0)) {
     for (int w = tm.tid; w < 4 * chi * chi; w += tm.nt) tout[w] = 0.0;
     for (int w = tm.tid; w < Dn; w += tm.nt) lamg[w] = 0.0;
-    if (tm.tid == 0) a.logacc[(int64_t)b * a.nslots + S + gd.bond] = -INFINITY;
+    if (tm.tid == 0) {
+      a.logacc[(int64_t)b * a.nslots + S + gd.bond] = -INFINITY;
+      if (non_finite(s0)) mark_non_finite(a, b);
+    }
     return;
   }
   if (rec) {

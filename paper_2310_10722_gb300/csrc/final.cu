@@ -91,16 +91,16 @@ __device__ void build_F(const Team& tm, const FinalArgs& fa, int b, int x, int y
 }
 
 // The cut of M = MT^T (m x n) by cut.cuh: the left vectors into An, the unscaled
-// carry into Cn.  Returns the number of states kept (0: the matrix is zero), or -1 when the scratch
-// does not hold the paths (the caller then takes the plain Jacobi of the recorded cuts).
+// carry into Cn.  Returns the number of states kept (0: the matrix is zero, or *s0 says not finite), or -1
+// when the scratch does not hold the paths (the caller then takes the plain Jacobi of the recorded cuts).
 // Scratch: shared memory (`pool` bytes at `sp`) as far as it goes, then the W, Q and R regions.
 static __device__ __noinline__ int cut(Team tm, const FinalArgs& fa, const double* MT, int ldm, int m, int n,
                                        double* work, double* W, double* An, double* Cn, unsigned char* sp, int64_t pool,
                                        int* slots, double (*sums)[32], double* trunc, double* s0) {
   const int q = m < n ? m : n, cm = fa.chi_mps, kk = cm < q ? cm : q;
   const int ex = cut_max_exponent(tm, MT, ldm, n, m, slots) - 1023;
-  if (ex == -1023) return 0;
-  *s0 = ldexp(1.0, ex);
+  *s0 = ldexp(1.0, ex);   // infinite for an infinity or NaN in the matrix (ex = 1024)
+  if (ex == -1023 || ex == 1024) return 0;
   if (m == 1) {
     // one state (outside the occupied grid): U = 1, carry = M
     for (int w = tm.tid; w < n; w += tm.nt) Cn[w] = MT[w];
@@ -239,6 +239,10 @@ __global__ void __launch_bounds__(NT, MINB) k_final(FinalArgs fa) {
   __shared__ double trunc_s[2];   // largest and summed discarded fraction of the cuts
   __shared__ double sum_s[2][32];
   const int nx = fa.nx, ny = fa.ny;
+  if (isnan(fa.logacc[(int64_t)b * fa.nslots + fa.slot])) {   // mark_non_finite
+    if (tm.tid < 2) fa.Z[(int64_t)b * 2 + tm.tid] = NAN;
+    return;
+  }
   if (tm.tid == 0) { logsum_s = 0.0; trunc_s[0] = 0.0; trunc_s[1] = 0.0; }
   for (int x = tm.tid; x < nx; x += tm.nt) {
     mdim[0][x][0] = 1; mdim[0][x][1] = 1; mdim[0][x][2] = (x == nx - 1) ? 2 : 1;
@@ -377,7 +381,7 @@ __global__ void __launch_bounds__(NT, MINB) k_final(FinalArgs fa) {
           }
         }
         if (k == 0) {
-          if (tm.tid == 0) logsum_s = -INFINITY;
+          if (tm.tid == 0) logsum_s += non_finite(s0) ? NAN : -INFINITY;
           for (int w = tm.tid; w < m; w += tm.nt) An[w] = R(0);
           for (int w = tm.tid; w < n; w += tm.nt) Cn[w] = R(0);
           if (tm.tid == 0) { mdim[cur ^ 1][x][0] = cJ; mdim[cur ^ 1][x][1] = U; mdim[cur ^ 1][x][2] = 1; }
@@ -440,7 +444,7 @@ __global__ void __launch_bounds__(NT, MINB) k_final(FinalArgs fa) {
               frexp(double(mx), &e2);
               logsum_s += double(e2) * 0.69314718055994530942;
             } else {
-              logsum_s = -INFINITY;
+              logsum_s += -INFINITY;
             }
             slam[0] = mx > R(0) ? R(ldexp(1.0, -e2)) : R(0);
             if (rs) { rs[9] = m; rs[10] = n; rs[12] = e2; }

@@ -82,9 +82,7 @@ __device__ __forceinline__ void local_site(const SweepArgs& a, const LocalDesc& 
 #pragma unroll
     for (int i = 0; i < P; ++i) {
       const unsigned hi = (unsigned)__double2hiint(v[i]) & 0x7FFFFFFFu, lo = (unsigned)__double2loint(v[i]);
-      // a NaN does not count (as in fmax); a subnormal value counts by its presence
-      const bool nan = hi > 0x7FF00000u || (hi == 0x7FF00000u && lo != 0u);
-      if (!nan) mx = max(mx, hi | (unsigned)(hi == 0u && lo != 0u));
+      mx = max(mx, hi | (unsigned)(hi == 0u && lo != 0u));   // a subnormal value counts by its presence
     }
   };
   double kept[KEEP][P];
@@ -109,10 +107,10 @@ __device__ __forceinline__ void local_site(const SweepArgs& a, const LocalDesc& 
   for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mx = max(mx, red[w]);
   int e2 = 0;
   const bool nz = mx > 0u;
-  const bool plain = mx >= 0x00100000u && mx < 0x7FF00000u;   // normal: mx = f 2^e2, f in [1/2, 1)
-  if (plain) e2 = (int)(mx >> 20) - 1022;
-  if (nz && !plain) {
-    // subnormal or infinite: as frexp of the value itself
+  const bool over = mx >= 0x7FF00000u;   // infinity or NaN
+  if (mx >= 0x00100000u && !over) e2 = (int)(mx >> 20) - 1022;   // normal: mx = f 2^e2, f in [1/2, 1)
+  if (nz && mx < 0x00100000u) {
+    // subnormal: as frexp of the value itself
     double m2 = 0.0;
     for (int r = threadIdx.x; r < d.rest; r += blockDim.x) {
       double v[P];
@@ -145,6 +143,7 @@ __device__ __forceinline__ void local_site(const SweepArgs& a, const LocalDesc& 
   if (threadIdx.x == 0) {
     double* la = a.logacc + (int64_t)b * a.nslots + s;
     *la += nz ? double(e2) * 0.69314718055994530942 : -INFINITY;
+    if (over || non_finite(sc)) mark_non_finite(a, b);   // sc: no factor scales a value below 2^-1024 up
     if (a.rec_sc) a.rec_sc[(int64_t)b * gridDim.x + s] = sc;
   }
 }

@@ -54,6 +54,16 @@ __device__ __forceinline__ const Override* vshot_ovr(const VShot* vs, const Over
   return (o->kind == kind && o->target == target) ? o : nullptr;
 }
 
+// A non-finite value (an overflow, or what follows from one) makes its shot's result NaN, reported by
+// td_network_check.  It is marked where it arises, with a NaN in the shot's last log-scale slot, which the
+// sweep does not use otherwise: further on it may meet zeros that are left out instead of multiplied (the rows and
+// columns that a truncation dropped), and the result would look like a number.
+__device__ __forceinline__ bool non_finite(double x) { return ((unsigned)__double2hiint(x) & 0x7FF00000u) == 0x7FF00000u; }
+__device__ __forceinline__ bool non_finite(float x) { return (__float_as_uint(x) & 0x7F800000u) == 0x7F800000u; }
+__device__ __forceinline__ void mark_non_finite(const SweepArgs& a, int b) {
+  a.logacc[(int64_t)b * a.nslots + a.nslots - 1] = __longlong_as_double(0x7FF8000000000000ll);
+}
+
 constexpr size_t kFinalStaticSmem = 8 * 1024;   // bound of k_final's own shared arrays
 
 struct FinalArgs {
