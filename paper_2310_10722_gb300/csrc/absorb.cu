@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "gramnum.cuh"
 #include "sweep.cuh"
 #include "tc.cuh"
 
@@ -838,17 +839,7 @@ __device__ __forceinline__ void tc_slices64(double v0, double v1, int E, uint32_
 }
 }  // namespace
 
-// |x| as an FP32 value truncated from the bit pattern (no FP64 instruction); big: out of FP32 range.
 namespace {
-__device__ __forceinline__ float tc_abs32(double x, bool& big) {
-  const unsigned hi = (unsigned)__double2hiint(x) & 0x7FFFFFFFu, lo = (unsigned)__double2loint(x);
-  big |= hi >= (1023u + 100u) << 20;
-  return hi < (1023u - 126u) << 20 ? 0.f : __uint_as_float(__funnelshift_l(lo, hi - (896u << 20), 3));
-}
-__device__ __forceinline__ float tc_abs32(float x, bool& big) {
-  big |= !(fabsf(x) < 1.2676506e30f);
-  return fabsf(x);
-}
 // The FP64 value of an FP32 integer, from its bit pattern.
 __device__ __forceinline__ double tc_widen(float v) {
   const unsigned b = __float_as_uint(v);
@@ -956,28 +947,29 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_gram_tc(SweepArgs a, const Ga
       return at | t << 30;
     };
     // 1. column bounds.  Only the exponent of a bound is used, so FP32 values within 2^-19 of the FP64
-    // ones decide it unless a bound comes that close to a power of two (then, or out of FP32 range, the
-    // bounds are formed as defined).
+    // ones decide it unless a bound comes that close to a power of two (then, or where a value or a row
+    // weight is out of FP32's range, the bounds are formed as defined).
     {
       float cm[DPAD];
-      bool big = false;
+      bool out = false;
 #pragma unroll
       for (int c = 0; c < DPAD; ++c) cm[c] = 0.f;
       for (int t = below(r_begin) + tid, t1 = below(r_end); t < t1; t += kTcThreads) {
         float w;
         const int ra = row(t, w, lam32), pr = ra >> 30, at = ra & 0x3FFFFFFF;
+        tc_weight32(w, out);
         const T* plo = gin + pg.lo(pr) * SZ + at;
         const T* phi = gin + pg.hi(pr) * SZ + at;
 #pragma unroll
         for (int c = 0; c < DPAD; ++c)
-          if (c < D) cm[c] = fmaxf(cm[c], (tc_abs32(plo[(int64_t)c * inner], big) + tc_abs32(phi[(int64_t)c * inner], big)) * w);
+          if (c < D) cm[c] = fmaxf(cm[c], (tc_abs32(plo[(int64_t)c * inner], out) + tc_abs32(phi[(int64_t)c * inner], out)) * w);
       }
 #pragma unroll
       for (int c = 0; c < DPAD; ++c) {
         const unsigned v = __reduce_max_sync(0xffffffffu, __float_as_uint(cm[c]));
         if (lane == 0 && v > 0u) atomicMax(&colbits[c], v);
       }
-      if (big) amb_s = 1;
+      if (out) amb_s = 1;
     }
     __syncthreads();
     if (tid < DPAD) {
