@@ -31,6 +31,7 @@
 #include <cmath>
 
 #include "gramnum.cuh"
+#include "launch.cuh"
 #include "sweep.cuh"
 #include "tc.cuh"
 
@@ -651,15 +652,15 @@ static cudaError_t gram_launch(const SweepArgs& a, const GateDesc* g, int count,
   const unsigned blocks = (unsigned)((n_jobs + wpb - 1) / wpb);
   const size_t smem = (size_t)wpb * kMaxBonds * a.chi * sizeof(double);
   if constexpr (DMAX == 8) {
-    cudaError_t e = cudaFuncSetAttribute(k_gram_sym8<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared_memory<k_gram_sym8<T>>();
     if (e != cudaSuccess) return e;
     k_gram_sym8<T><<<blocks, wpb * 32, smem, st>>>(a, g, gram, n_jobs, nchunk, chunk_rows);
   } else if constexpr (DMAX == 16) {
-    cudaError_t e = cudaFuncSetAttribute(k_gram_sym16<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared_memory<k_gram_sym16<T>>();
     if (e != cudaSuccess) return e;
     k_gram_sym16<T><<<blocks, wpb * 32, smem, st>>>(a, g, gram, n_jobs, nchunk, chunk_rows);
   } else {
-    cudaError_t e = cudaFuncSetAttribute(k_gram<T, DMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared_memory<k_gram<T, DMAX>>();
     if (e != cudaSuccess) return e;
     k_gram<T, DMAX><<<blocks, wpb * 32, smem, st>>>(a, g, gram, n_jobs, nchunk, chunk_rows);
   }
@@ -691,7 +692,7 @@ static cudaError_t update_launch(const SweepArgs& a, const GateDesc* g, int coun
   const int64_t n_jobs = sides * nchunk;
   const unsigned blocks = (unsigned)((n_jobs + wpb - 1) / wpb);
   const size_t smem = (size_t)wpb * 2 * DMAX * DMAX * sizeof(double);
-  e = cudaFuncSetAttribute(k_update<T, DMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = allow_shared_memory<k_update<T, DMAX>>();
   if (e != cudaSuccess) return e;
   k_update<T, DMAX><<<blocks, wpb * 32, smem, st>>>(a, g, tbuf, n_jobs, nchunk);
   return cudaGetLastError();
@@ -1227,7 +1228,7 @@ static cudaError_t gram_tc_launch(const SweepArgs& a, const GateDesc* g, int cou
   const int64_t n_jobs = (int64_t)count * a.B * 2 * nchunk;
   if (n_jobs == 0) return cudaSuccess;
   const size_t smem = tc_smem_bytes<DPAD>(a.chi);
-  cudaError_t e = cudaFuncSetAttribute(k_gram_tc<T, DPAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_shared_memory<k_gram_tc<T, DPAD>>();
   if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

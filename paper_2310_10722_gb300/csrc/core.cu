@@ -25,6 +25,7 @@
 #include <cfloat>
 #include <cmath>
 
+#include "launch.cuh"
 #include "sweep.cuh"
 #include "team.cuh"
 
@@ -482,7 +483,7 @@ cudaError_t launch_core2(const SweepArgs& a, const GateDesc* g, int count, int D
   int items = 128 / tt;
   while (items > 1 && n_items <= (int64_t)kCoreSpread * nsm * items / 4) items /= 2;
   const size_t smem = (size_t)items * CoreSmem::bytes(Dm);
-  e = cudaFuncSetAttribute(k_core2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = allow_shared_memory<k_core2>();
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)((n_items + items - 1) / items);
   k_core2<<<blocks, 128, smem, st>>>(a, g, gram, tbuf, S, (int)n_items, items, tt, Dm, precond ? 1 : 0);

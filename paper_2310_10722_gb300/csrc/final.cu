@@ -22,6 +22,7 @@
 #include <mutex>
 
 #include "cut.cuh"
+#include "launch.cuh"
 #include "sweep.cuh"
 #include "team.cuh"
 
@@ -544,7 +545,7 @@ static cudaError_t final_launch(const FinalArgs& f, cudaStream_t st) {
   a.cut_smem = (int32_t)pool;
   const size_t smem = (size_t)(wk + pool);
   if (smem > 0) {
-    e = cudaFuncSetAttribute(k_final<T, R, NT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_shared_memory<k_final<T, R, NT, MINB>>();
     if (e != cudaSuccess) return e;
   }
   k_final<T, R, NT, MINB><<<f.B, NT, smem, st>>>(a);

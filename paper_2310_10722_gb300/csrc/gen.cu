@@ -9,6 +9,7 @@
 #include <cmath>
 
 #include "gen.cuh"
+#include "launch.cuh"
 
 namespace td {
 
@@ -81,7 +82,7 @@ cudaError_t launch_gen_rows(const GenRowsArgs& g, cudaStream_t st) {
   const unsigned blocks = (unsigned)((g.B + kGenWarps - 1) / kGenWarps);
   const size_t smem = (size_t)kGenWarps * g.words * sizeof(unsigned long long);
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_gen_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared_memory<k_gen_rows>();
     if (e != cudaSuccess) return e;
   }
   k_gen_rows<<<blocks, kGenWarps * 32, smem, st>>>(g);
