@@ -305,15 +305,11 @@ __global__ void k_core2(SweepArgs a, const GateDesc* __restrict__ gates, const d
   // pivot tolerance per block: gram_cutoff times the side's largest diagonal (< 0: empty)
   if (tm.tid < 4) {
     const int side = tm.tid / 2;
-    double e = 0.0;
-    bool over = false;
+    long long top = 0;   // on the bit patterns: NaN above infinity above the finite values, negative ones below 0
     for (int blk = 2 * side; blk < 2 * side + 2; ++blk)
-      for (int j = 0; j < D; ++j) {
-        const double g = RG[blk * DD + j * D + j];
-        over |= non_finite(g);
-        e = fmax(e, g);
-      }
-    if (over) mark_non_finite(a, b);
+      for (int j = 0; j < D; ++j) top = max(top, __double_as_longlong(RG[blk * DD + j * D + j]));
+    const double e = __longlong_as_double(top);
+    if (non_finite(e)) mark_non_finite(a, b);
     sm.sv[tm.tid] = e > 0.0 ? a.gram_cutoff * e : -1.0;
   }
   tm.sync();
