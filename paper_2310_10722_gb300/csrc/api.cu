@@ -179,15 +179,9 @@ static void final_layout(td_network* net, int threads, bool allow_smem = true) {
   const int64_t mps_stride = ((int64_t)cm * Dm * cmx + 3) / 4 * 4;
   const int64_t mF = 2LL * Dm * Dm * Dm * Dm;
   net->fin.threads = threads;
-  int64_t mMT = 0, mV = 0;   // M^T (n x m) and V (m x m) with the bank-spreading leading dimensions
-  {
-    const int n_max = (int)(cmx * Dm * 2), m_max = cm * Dm;
-    for (int m = 1; m <= m_max; ++m) {
-      const int g = td::team_svd_group(threads, n_max, m);
-      mMT = std::max<int64_t>(mMT, (int64_t)m * td::bank_ld32(n_max, g));
-      mV = std::max<int64_t>(mV, (int64_t)m * td::bank_ld32(m, g));
-    }
-  }
+  // M^T (n x m) and V (m x m) with the bank-spreading leading dimensions
+  const int64_t mMT = td::final_mt_elems(threads, (int)(cmx * Dm * 2), cm * Dm);
+  int64_t mV = td::final_v_elems(threads, (int)(cmx * Dm * 2), cm * Dm);
   // columns of a cut's factor (cut_ldl)
   int64_t mR = 0;
   {
@@ -219,6 +213,7 @@ static void final_layout(td_network* net, int threads, bool allow_smem = true) {
   net->fin.w_W = wtake(mW);
   net->fin.W_elems = mW;
   net->fin.w_MT = wtake(mMT);
+  net->fin.MT_elems = mMT;
   net->fin.w_C0 = wtake(mC);
   net->fin.w_C1 = wtake(mC);
   net->fin.w_s = wtake(mS);

@@ -297,12 +297,12 @@ __global__ void __launch_bounds__(NT, MINB) k_final(FinalArgs fa) {
       tm.sync();
       // MT[(bb, r, q)][(j, u)] = sum_{l,p,d} T1[l][p][d][bb][j] F[p^q][l][r][d][u], stored
       // column-major: column (j, u) of MT is row (j, u) of M; leading dimensions chosen so
-      // the Jacobi lane groups of consecutive columns fall on disjoint banks
+      // the Jacobi lane groups of consecutive columns fall on disjoint banks where they fit
       const int nF = L * Rr * aD * U;
       const int m = cJ * U, n = aR * Rr * 2;
       const int pc = fd[4];   // 0: F[1] is zero, so only p = q contributes (half the products)
-      const int ldm = bank_ld32(n, team_svd_group(tm.nt, n, m));
-      const int ldv = bank_ld32(m, team_svd_group(tm.nt, n, m));
+      const int lanes = team_svd_group(tm.nt, n, m);
+      const int ldm = final_ld(n, lanes, m, fa.MT_elems), ldv = final_ld(m, lanes, m, fa.W_elems);
       for (int w = tm.tid; w < m * n; w += tm.nt) {
         const int c = w / m, ju = w % m;      // consecutive lanes: consecutive u (F) and ju (MT)
         const int q = c % 2, r = (c / 2) % Rr, bb = c / (2 * Rr);

@@ -81,7 +81,7 @@ struct FinalArgs {
   int64_t work_elems;        // work region size (elements)
   int64_t w_F, w_W, w_MT, w_C0, w_C1, w_s, w_ord;   // offsets inside the work region
   int64_t w_Q, w_R;          // scratch of the cuts: a copy of the matrix, the columns of its factor
-  int64_t W_elems;           // size of the W region (elements)
+  int64_t W_elems, MT_elems; // sizes of the W and M^T regions (elements)
   int32_t use_smem;          // work region in dynamic shared memory
   int32_t cut_need;          // bytes of shared memory the largest cut that truncates can use
   int32_t cut_smem;          // bytes of it given to this launch
