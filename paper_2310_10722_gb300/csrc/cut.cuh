@@ -1015,10 +1015,9 @@ static __device__ __noinline__ int cut_qrcp_cols(Team tm, double* X, int m, int 
 
 // Cut of rank <= most (nothing to truncate): X = M (m x n, row-major; destroyed); U (m x r) into An
 // (row-major), the carry R (r x n) into Cn; Qs: most x m scratch, vr: 4 most, nrm: n, all FP64.  Returns
-// r, or -1 when more than `most` pivots lie above the cutoff.  *rest: the largest squared column norm
-// left out over the largest of all.
+// r, or -1 when more than `most` pivots lie above the cutoff.
 static __device__ __noinline__ int cut_rank(Team tm, double* X, int m, int n, int most, double cutoff, double* An, double* Cn,
-                                            double* Qs, double* vr, double* nrm, CutBuf& b, double* s0, double* rest) {
+                                            double* Qs, double* vr, double* nrm, CutBuf& b, double* s0) {
   double left;
   const int q = m < n ? m : n;
   const int r = cut_qrcp_cols(tm, X, m, n, cutoff * cutoff, most < q ? most : q, vr, nrm, b.taken, b.keys, left);
@@ -1048,7 +1047,6 @@ static __device__ __noinline__ int cut_rank(Team tm, double* X, int m, int n, in
   }
   for (int w = tm.tid; w < m * r; w += tm.nt) An[w] = Qs[(size_t)(w % r) * m + w / r];
   *s0 = fabs(vr[2]);
-  *rest = r < q ? left : 0.0;
   tm.sync();
   return r;
 }

@@ -91,6 +91,36 @@ __device__ void build_F(const Team& tm, const FinalArgs& fa, int b, int x, int y
   tm.sync();
 }
 
+// Discarded fraction of a cut: |M - U U^T M|^2 over |M|^2, entry by entry (no cancellation); M = MT^T, U (m x k,
+// row-major), C = U^T M (k x n).
+static __device__ __noinline__ double cut_discarded(Team tm, const double* MT, int ldm, int m, int n, const double* U,
+                                                    const double* C, int k, double (*sums)[32]) {
+  double disc = 0.0, tot = 0.0;
+  for (int w = tm.tid; w < m * n; w += tm.nt) {
+    const int c = w / n, i = w % n;
+    const double a = MT[(size_t)c * ldm + i];
+    double d = a;
+    for (int j = 0; j < k; ++j) d -= C[(size_t)j * n + i] * U[c * k + j];
+    disc += d * d;
+    tot += a * a;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    disc += __shfl_xor_sync(0xffffffffu, disc, o);
+    tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  }
+  if ((tm.tid & 31) == 0) {
+    sums[0][tm.tid >> 5] = disc;
+    sums[1][tm.tid >> 5] = tot;
+  }
+  tm.sync();
+  disc = tot = 0.0;
+  for (int w = 0; w < tm.nt / 32; ++w) {
+    disc += sums[0][w];
+    tot += sums[1][w];
+  }
+  return disc / tot;
+}
+
 // The cut of M = MT^T (m x n) by cut.cuh: the left vectors into An, the unscaled
 // carry into Cn.  Returns the number of states kept (0: the matrix is zero, or *s0 says not finite), or -1
 // when the scratch does not hold the paths (the caller then takes the plain Jacobi of the recorded cuts).
@@ -143,32 +173,7 @@ static __device__ __noinline__ int cut(Team tm, const FinalArgs& fa, const doubl
         for (int w = tm.tid; w < m * k; w += tm.nt) An[w] = cb.V[w];
         if (vs)
           for (int w = tm.tid; w < k * n; w += tm.nt) Cn[w] = cb.P[w];
-        if (fa.stats) {   // |M - U U^T M|^2 over |M|^2, entry by entry (no cancellation)
-          double disc = 0.0, tot = 0.0;
-          for (int w = tm.tid; w < m * n; w += tm.nt) {
-            const int c = w / n, i = w % n;
-            const double a = MT[(size_t)c * ldm + i];
-            double d = a;
-            for (int j = 0; j < k; ++j) d -= cb.P[(size_t)j * n + i] * cb.V[c * k + j];
-            disc += d * d;
-            tot += a * a;
-          }
-          for (int o = 16; o > 0; o >>= 1) {
-            disc += __shfl_xor_sync(0xffffffffu, disc, o);
-            tot += __shfl_xor_sync(0xffffffffu, tot, o);
-          }
-          if ((tm.tid & 31) == 0) {
-            sums[0][tm.tid >> 5] = disc;
-            sums[1][tm.tid >> 5] = tot;
-          }
-          tm.sync();
-          disc = tot = 0.0;
-          for (int w = 0; w < tm.nt / 32; ++w) {
-            disc += sums[0][w];
-            tot += sums[1][w];
-          }
-          rest = disc / tot;
-        }
+        if (fa.stats) rest = cut_discarded(tm, MT, ldm, m, n, cb.V, cb.P, k, sums);
       }
     }
   }
@@ -183,7 +188,8 @@ static __device__ __noinline__ int cut(Team tm, const FinalArgs& fa, const doubl
       double* X = xs ? Qs + (size_t)kk * m : Q;
       for (int w = tm.tid; w < m * n; w += tm.nt) X[w] = MT[(size_t)(w / n) * ldm + w % n];
       tm.sync();
-      k = cut_rank(tm, X, m, n, kk, fa.svd_cutoff, An, Cn, Qs, vr, nrm, cb, s0, &rest);
+      k = cut_rank(tm, X, m, n, kk, fa.svd_cutoff, An, Cn, Qs, vr, nrm, cb, s0);
+      if (fa.stats && k > 0 && k < q) rest = cut_discarded(tm, MT, ldm, m, n, An, Cn, k, sums);
     }
   }
   if (k < 0) {
