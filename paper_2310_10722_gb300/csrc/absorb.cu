@@ -1,5 +1,6 @@
 // Gate absorption passes of the sweep (Sec. 4): the Gram pass and the update pass of the
-// simple update, one warp per (gate side, shot, row chunk).
+// simple update, over jobs of (gate side, shot, row chunk): one warp per job, one block in the Gram on the
+// tensor cores.
 //
 // The two-site gate (1-p) I x I + p X x X is applied by doubling its bond (see sweep.cu):
 // with Y = M[sigma_lo] + M[sigma_hi] and Z = M[sigma_lo] - M[sigma_hi] for each physical
@@ -11,12 +12,13 @@
 // Gamma_new[lo] = Y T0, Gamma_new[hi] = Z T1.
 //
 // A side tensor is [phys][outer][D][inner]; a row is (pair, outer index o, inner index i)
-// and holds D values at stride `inner`.  Each row is handled by LPR lanes; lane `sub` of a
-// row loads BPL = DMAX/LPR of its columns, and the full row is assembled in every lane of
-// the row by shuffles.  The Gram lane accumulates its BPL x DMAX block of G+ and of G- in
-// registers, summed over the warp at the end; the update lane produces BPL output columns.
-// No shared-memory staging of the data and no block-wide barrier.  Chunks of a long side
-// write separate partial Grams, summed in a fixed order by the core kernel (deterministic).
+// and holds D values at stride `inner`.  In the warps' passes each row is handled by LPR lanes; lane `sub`
+// of a row loads BPL = DMAX/LPR of its columns, and the full row is assembled in every lane of the row by
+// shuffles.  The Gram lane takes BPL neighbouring columns and accumulates its BPL x DMAX block of G+ and of
+// G- in registers, summed over the warp at the end; the update lane takes the columns sub, sub + LPR, ... and
+// produces as many output columns, from T+ and T- staged per warp in shared memory.  The rows are not
+// staged, and no barrier is block-wide.  Chunks of a long side write separate partial Grams, summed in a
+// fixed order by the core kernel (deterministic).
 //
 // Precision.  Both passes compute in FP64 for both storage types (FP32 storage is read,
 // widened, and the update's result rounded back): the Gram's small eigenvalues come from

@@ -56,7 +56,7 @@ struct td_network {
   td::FinalArgs fin{};
   int64_t fscr_elems = 0;       // final-contraction scratch per shot (largest candidate layout)
   int smem_optin = 0, smem_sm = 0;
-  int32_t chunk_rows = td::kChunkRows;   // rows per Gram / update job
+  int32_t chunk_rows = td::kChunkRows;   // rows per Gram job
   size_t bytes = 0;
   int64_t launches_per_wave = 0;
   std::vector<void*> allocs;
@@ -202,6 +202,8 @@ static void final_layout(td_network* net, int threads, bool allow_smem = true) {
         mV = std::max<int64_t>(mV, (int64_t)n * td::bank_ld32(n, g));
       }
   }
+  // the Q region also keeps room for two square matrices: the scratch per shot decides which batches
+  // td_coset_logprob_static accepts
   const int64_t mP = (int64_t)(cm * Dm + 1) * cm * Dm, mT = (int64_t)cm * Dm * cm * Dm;
   const int64_t mW = std::max<int64_t>({(int64_t)cm * Dm * 2 * Dm * cmx, mV, mR});
   const int64_t mC = (int64_t)cm * cmx * Dm * 2;

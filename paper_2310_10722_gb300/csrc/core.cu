@@ -72,7 +72,7 @@ __device__ __forceinline__ void load_gram(const Team& tm, const double* gram, in
   }
 }
 
-// FP64 one-sided Jacobi sweeps (as team_svd_onesided with V given) of the items of one block of four
+// FP64 one-sided Jacobi sweeps (as team_svd_onesided, but V is given and updated) of the items of one block of four
 // warps in lock step: up to four items of one-warp teams, two of two, one of four.
 //
 // What bounds it: an FP64 instruction holds its warp's scheduler for 64 cycles (and the SM's FP64
@@ -84,8 +84,9 @@ __device__ __forceinline__ void load_gram(const Team& tm, const double* gram, in
 // four warps row by row; a pair's three sums are reduced side by side (3 instead of 6 instructions for
 // 4 lanes), or, when a block has fewer items than warps, by different warps.  The same operations in
 // the same order on every value: bit for bit the result of team_svd_onesided.  Measured (core time of
-// a decode, before -> with this; the angles' quotients in integers, ieee.cuh, took off another 6-11 %): rotated d9 chi 8, 1000 shots mixed 178 -> 129 ms, 152 shots FP64 66 -> 47
-// ms; d7 FP64, 48 shots 29.4 -> 18.9 ms; d5, 37 shots 10.1 -> 7.4 ms.
+// a decode, before -> with this; the angles' quotients in integers, ieee.cuh, took off another 6-11 %):
+// rotated d9 chi 8, 1000 shots mixed 178 -> 129 ms, 152 shots FP64 66 -> 47 ms; d7 FP64, 48 shots
+// 29.4 -> 18.9 ms; d5, 37 shots 10.1 -> 7.4 ms.
 // Not done: keeping the squared norms of columns that did not rotate (a twelfth fewer FP64 instructions):
 // 121.5 -> 120.5 ms with a full chip, but 6.8 -> 7.2 ms for d5, 37 shots, where a step is a chain.
 struct GroupJacobi {

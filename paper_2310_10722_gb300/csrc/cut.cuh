@@ -504,10 +504,10 @@ static __device__ __noinline__ void block_svd_onesided(Team tm, double* A, int l
   }
 }
 
-// FP32 one-sided Jacobi of the r columns of L, without V, four rows per load and two per instruction: columns padded with zeros to a multiple
-// of 32 rows (rows32), ld cut_ld32.  What bounds it is instructions (18 per 4 rows of a pair against
-// ~80 one by one) and the latency of a step (~350 cycles); N4 loads per lane and column stay in
-// registers, N4 = 0 reads them twice.
+// FP32 one-sided Jacobi of the r columns of L, without V, four rows per load and two per instruction:
+// columns padded with zeros to a multiple of 32 rows (rows32), ld cut_ld32.  What bounds it is
+// instructions (18 per 4 rows of a pair against ~80 one by one) and the latency of a step (~350 cycles);
+// N4 loads per lane and column stay in registers, N4 = 0 reads them twice.
 template <int N4>
 __device__ __noinline__ void cut_jacobi32(Team tm, float* L, int ldl, int rows32, int r, int g, int* flag) {
   constexpr int N = N4 > 0 ? N4 : 1;
@@ -714,7 +714,7 @@ static __device__ __noinline__ void cut_orthonormalise(Team tm, const double* V,
   tm.sync();
 }
 
-// Leading dimension of the columns that cut_jacobi turns: = lanes per pair mod 32 at full rank, which
+// Leading dimension of the columns that cut_jacobi64 turns: = lanes per pair mod 32 at full rank, which
 // puts the lane groups of consecutive pairs on different banks.
 __host__ __device__ __forceinline__ int cut_ldl(int nt, int m) { return bank_ld32(m, team_svd_group(nt, m, m)); }
 // The same for four-row loads: eight lanes' 128 bytes on different banks (a multiple of 4; below
@@ -946,7 +946,9 @@ constexpr double kCutRankCutoff = 1e-11;
 // Householder QR with column pivoting of the m x n matrix X (row-major, ld n; destroyed), m <= 64 or so:
 // a thread per column, so that every FP64 instruction works on 32 columns (a column per warp leaves
 // most lanes idle on the few rows of a cut that does not truncate).  Two barriers per step: pivot;
-// reflector (formed by one warp).  Stop and vr as cut_qrcp, the reflector's tail in column piv_j; nrm:
+// reflector (formed by one warp).  Stops at the first pivot norm^2 <= abs2 times that of the first, or after
+// `most` steps (*left: the squared norm of the pivot that it stopped at, over the first's); vr[4 j ..]: the
+// reflector's head, 2 / v.v, R[j][j] and the pivot column of step j, the reflector's tail in that column; nrm:
 // n, keys: nw.
 static __device__ __noinline__ int cut_qrcp_cols(Team tm, double* X, int m, int n, double abs2, int most, double* vr,
                                                  double* nrm, unsigned char* taken, unsigned* keys, double& left) {

@@ -14,9 +14,9 @@
 // sums and FP32 singular vectors err by ~eps32 times the majority coset's weight, a relative
 // error of ~eps32 exp(margin) on the minority coset.  The cuts are those of cut.cuh, to FP64
 // accuracy on every path; the gradient pass's recorded forward takes a one-sided Jacobi SVD of
-// M^T with V accumulated (its records are M^T V and V), bit for bit the same whatever the block: the
-// adjoint divides by differences of singular values, so another rounding here moves single entries of
-// the gradient by up to 1e-6.
+// M^T with V accumulated (its records are M^T V and V), with the rounding of team_svd_onesided for a block
+// of that size: the adjoint divides by differences of singular values, so another rounding here moves single
+// entries of the gradient by up to 1e-6.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(NT, MINB) k_final(FinalArgs fa) {
               double* buf = reinterpret_cast<double*>(smem_raw + (fa.use_smem ? fa.work_elems * sizeof(R) : 0));
               block_svd_onesided(tm, MT, ldm, n, m, V, ldv, buf, reinterpret_cast<int*>(buf + 5 * half), meta + 2, 40);
             } else {
-              team_svd_onesided<R>(tm, MT, ldm, n, m, V, ldv, meta + 7, 40, true);
+              team_svd_onesided<R>(tm, MT, ldm, n, m, V, ldv, meta + 7, 40);
             }
           }
           team_col_norms<R>(tm, MT, ldm, n, m, sv);

@@ -5,8 +5,8 @@
 // Jacobi rotations are a chain of two divisions and a square root.  Here each takes ~60 integer instructions
 // and none in FP64.  Measured (core time of a decode): rotated d9 chi 8, 1000 shots 129.0 -> 121.5 ms, its FP64 152
 // shots 47.4 -> 43.5, rotated d7 FP64, 48 shots 18.9 -> 16.7, rotated d5, 37 shots 7.37 -> 6.80; the sweep of
-// rotated d9 chi 16, 16 shots 128 -> 123 ms, a gradient 185 -> 179 ms.  Both are correctly rounded, as IEEE 754 defines the operations, so the values are
-// those of `/` and sqrt() bit for bit.
+// rotated d9 chi 16, 16 shots 128 -> 123 ms, a gradient 185 -> 179 ms.  Both are correctly rounded, as
+// IEEE 754 defines the operations, so the values are those of `/` and sqrt() bit for bit.
 //
 // How: Newton's iteration from an FP32 estimate (relative error below 2^-21), one cubic step in fixed
 // point (1 / (1 - e) = 1 + e + e^2 + O(e^3), (1 - e)^(-1/2) = 1 + e / 2 + 3 e^2 / 8 + O(e^3)), which leaves an error below

@@ -68,87 +68,13 @@ __device__ __forceinline__ void team_rr_pair(int k, int i, int ne, int& p, int& 
   }
 }
 
-// Pivoted Cholesky of the symmetric positive semi-definite D x D matrix G (row-major,
-// leading dimension ldg; destroyed), D <= 32.  Pivot k is the largest remaining diagonal
-// entry; the factorisation stops when it is <= tol.  On return rows 0..r-1 of Rf (ld ldr)
-// hold the factor in the original column order -- G ~= Rf^T Rf, Rf[i][piv[j]] = 0 for
-// j < i -- and piv[0..r) the pivot columns.  `shr` is 2 ints of team-shared scratch.
-// Returns the rank r.
-template <typename R>
-__device__ int team_pchol(const Team& tm, R* G, int ldg, int D, R tol, R* Rf, int ldr, int* piv, int* shr) {
-  uint32_t done = 0;
-  int r = 0;
-  for (int k = 0; k < D; ++k) {
-    if (tm.tid < 32) {
-      const int lane = tm.tid;
-      R v = (lane < D && !((done >> lane) & 1u)) ? G[lane * ldg + lane] : R(-1);
-      int idx = lane;
-      for (int o = 16; o > 0; o >>= 1) {
-        const R v2 = __shfl_xor_sync(0xffffffffu, v, o);
-        const int i2 = __shfl_xor_sync(0xffffffffu, idx, o);
-        if (v2 > v || (v2 == v && i2 < idx)) {
-          v = v2;
-          idx = i2;
-        }
-      }
-      if (lane == 0) {
-        shr[0] = idx;
-        shr[1] = (v > tol) ? 1 : 0;
-      }
-    }
-    tm.sync();
-    const int p = shr[0];
-    if (!shr[1]) break;
-    const R rkk = sqrt(G[p * ldg + p]);
-    const R inv = R(1) / rkk;
-    for (int c = tm.tid; c < D; c += tm.nt) {
-      R v;
-      if (c == p)
-        v = rkk;
-      else if ((done >> c) & 1u)
-        v = R(0);
-      else
-        v = G[p * ldg + c] * inv;
-      Rf[k * ldr + c] = v;
-    }
-    if (tm.tid == 0) piv[k] = p;
-    done |= 1u << p;
-    tm.sync();
-    for (int w = tm.tid; w < D * D; w += tm.nt) {
-      const int a = w / D, c = w % D;
-      if (((done >> a) & 1u) || ((done >> c) & 1u)) continue;
-      G[a * ldg + c] -= Rf[k * ldr + a] * Rf[k * ldr + c];
-    }
-    tm.sync();
-    r = k + 1;
-  }
-  return r;
-}
-
-// Right inverse of the pivoted factor: Ri (D x r, ld ldi) with Rf Ri = I_r, nonzero only
-// in the pivot rows: Ri[piv[i]][j] = (R11^-1)[i][j], R11[i][j] = Rf[i][piv[j]] upper
-// triangular.  One column of R11^-1 per thread, by back substitution.
-template <typename R>
-__device__ void team_pchol_rinv(const Team& tm, const R* Rf, int ldr, const int* piv, int r, int D, R* Ri,
-                                int ldi) {
-  for (int w = tm.tid; w < D * r; w += tm.nt) Ri[(w / r) * ldi + (w % r)] = R(0);
-  tm.sync();
-  for (int j = tm.tid; j < r; j += tm.nt) {
-    Ri[piv[j] * ldi + j] = R(1) / Rf[j * ldr + piv[j]];
-    for (int i = j - 1; i >= 0; --i) {
-      R s = R(0);
-      for (int l = i + 1; l <= j; ++l) s += Rf[i * ldr + piv[l]] * Ri[piv[l] * ldi + j];
-      Ri[piv[i] * ldi + j] = -s / Rf[i * ldr + piv[i]];
-    }
-  }
-  tm.sync();
-}
-
-// Four independent pivoted Cholesky factorisations (as team_pchol) run concurrently: the
-// team is split into four lane segments of seg = nt/4 lanes (D <= seg <= 32); segment b
-// factors the D x D block G + b*bstride into Rf + b*bstride (ld D), with its pivots and the
-// reciprocals of R11's diagonal (from one rsqrt per pivot) in piv/dinv + b*pstride and its
-// rank in rank[b] (team-shared).  tol[b] < 0 marks an empty block (rank 0).  Pivot
+// Four independent pivoted Cholesky factorisations of symmetric positive semi-definite D x D blocks run
+// concurrently: the team is split into four lane segments of seg = nt/4 lanes (D <= seg <= 32); segment b
+// factors the block G + b*bstride (row-major, destroyed) into Rf + b*bstride (ld D).  Pivot k is the largest
+// remaining diagonal entry; the factorisation stops when it is <= tol[b] (< 0 marks an empty block, rank 0).
+// Rows 0..r-1 of the factor are in the original column order -- G ~= Rf^T Rf, Rf[i][piv[j]] = 0 for j < i --,
+// the pivot columns and the reciprocals of R11's diagonal (from one rsqrt per pivot) in piv/dinv + b*pstride,
+// the rank in rank[b] (team-shared).  Pivot
 // candidates are compared as bit patterns: non-negative doubles order as integers, and a
 // negative rounding residue loses to any admissible pivot.
 __device__ __forceinline__ void team_pchol4(const Team& tm, double* G, int D, int bstride, const double* tol,
@@ -212,9 +138,9 @@ __device__ __forceinline__ void team_pchol4(const Team& tm, double* G, int D, in
   tm.sync();
 }
 
-// Right inverses of the four factors of team_pchol4 (as team_pchol_rinv, multiplying by
-// the stored reciprocal diagonals): Ri + b*bstride is D x r_b (ld D); one (block, column)
-// per thread.
+// Right inverses of the four factors of team_pchol4: Ri + b*bstride is D x r_b (ld D) with Rf Ri = 1, nonzero
+// only in the pivot rows: Ri[piv[i]][j] = (R11^-1)[i][j], R11[i][j] = Rf[i][piv[j]] upper triangular, by back
+// substitution with the stored reciprocal diagonals; one (block, column) per thread.
 __device__ __forceinline__ void team_pchol_rinv4(const Team& tm, const double* Rf, int D, int bstride, const int* piv,
                                                  const double* dinv, int pstride, const int* rank, double* Ri) {
   for (int w = tm.tid; w < 4 * D * D; w += tm.nt) Ri[(w / (D * D)) * bstride + w % (D * D)] = 0.0;
@@ -281,16 +207,13 @@ __device__ __forceinline__ int team_pow2_floor(int x) {
 // A[c * lda + r]; an odd lda keeps the lanes of different column pairs on different shared
 // memory banks): on return the columns of A are mutually orthogonal, A_out = A_in V, with
 // V (n x n, column-major, ldv) orthogonal -- so the singular values are the column norms
-// of A_out and its normalised columns the left singular vectors.  With init_V false, V
-// holds an orthogonal matrix on entry and is updated as V <- V J.  `flag` is one int of
+// of A_out and its normalised columns the left singular vectors.  `flag` is one int of
 // team-shared scratch.  Returns the number of sweeps.
-// `tol`: convergence tolerance (<= 0: TeamTol<R>::rel()).
 template <typename R>
 __device__ int team_svd_onesided(const Team& tm, R* A, int lda, int m, int n, R* V, int ldv, int* flag,
-                                 int max_sweeps, bool init_V = true, R tol = R(0)) {
-  if (!(tol > R(0))) tol = TeamTol<R>::rel();
-  if (init_V)
-    for (int w = tm.tid; w < n * n; w += tm.nt) V[(w / n) * ldv + (w % n)] = (w / n == w % n) ? R(1) : R(0);
+                                 int max_sweeps) {
+  const R tol = TeamTol<R>::rel();
+  for (int w = tm.tid; w < n * n; w += tm.nt) V[(w / n) * ldv + (w % n)] = (w / n == w % n) ? R(1) : R(0);
   tm.sync();
   if (n < 2) return 0;
   const int ne = n + (n & 1), half = ne / 2;
@@ -424,18 +347,6 @@ __device__ inline double team_absmax(const Team& tm, const double* x, int ld, in
   return r;
 }
 
-// C (m x n) = A (m x k) B (k x n), all row-major with the given leading dimensions.
-template <typename R>
-__device__ __forceinline__ void team_gemm(const Team& tm, const R* A, int lda, const R* B, int ldb, R* C, int ldc,
-                                          int m, int n, int k) {
-  for (int w = tm.tid; w < m * n; w += tm.nt) {
-    const int i = w / n, j = w % n;
-    R s = R(0);
-    for (int l = 0; l < k; ++l) s += A[i * lda + l] * B[l * ldb + j];
-    C[i * ldc + j] = s;
-  }
-}
-
 // Start of a one-sided Jacobi SVD of A (m x n, column-major, lda) from an FP32 solve
 // (mixed-precision Jacobi): the FP32 Jacobi runs on a copy scaled to a largest entry of 1; its
 // right factor, re-orthogonalised in FP64 by one Newton-Schulz step V <- V (3I - V^T V) / 2, is applied
@@ -460,7 +371,7 @@ __device__ inline void svd_precond(const Team& tm, double* A, int lda, int m, in
     A32[c * la32 + r] = float(A[c * lda + r] * sc);
   }
   tm.sync();
-  team_svd_onesided<float>(tm, A32, la32, m, n, V32, lv32, flag, 30, true);
+  team_svd_onesided<float>(tm, A32, la32, m, n, V32, lv32, flag, 30);
   for (int w = tm.tid; w < n * n; w += tm.nt) {
     const int c = w / n, r = w % n;
     V[c * ldv + r] = double(V32[c * lv32 + r]);
