@@ -53,15 +53,22 @@ typedef enum {
 } td_status;
 
 typedef enum {
-  TD_FP64 = 0,   /* the plain FP64 GPU path: FP64 storage and arithmetic on the CUDA cores
-                    everywhere, every SVD an FP64 one-sided Jacobi */
+  TD_FP64 = 0,   /* the plain FP64 GPU path: FP64 storage and arithmetic on the CUDA cores, every
+                    SVD of a truncation core an FP64 one-sided Jacobi; the zip-up cuts as below */
   TD_FP32 = 1,   /* mixed precision with FP32 storage of the site tensors: the Gram pass on
                     the tcgen05 tensor cores (below), the update and site operators in FP64
-                    arithmetic, every SVD (truncation cores, zip-up cuts) FP32-preconditioned
-                    and finished by FP64 Jacobi sweeps, the final contraction and log-sum in
-                    FP64 */
+                    arithmetic, the SVDs of the truncation cores FP32-preconditioned and finished
+                    by FP64 Jacobi sweeps, the final contraction and log-sum in FP64 */
   TD_TC = 2      /* mixed precision with FP64 storage (the headline mixed path): as TD_FP32,
                     with the site tensors kept in FP64 */
+  /* The zip-up cuts, on every path: the products and the boundary MPS are FP64.  Where FP32
+   * resolves a cut -- which values are kept under both truncation rules, with room for FP32's
+   * error -- its kept space starts from an FP32 pivoted QR and Jacobi and is corrected by Newton
+   * steps with FP64 residuals until the residual is at FP64 rounding (below 5e-16 of the largest
+   * singular value, or below 2e-14 and no longer falling); the steps' corrections are FP32.  Every
+   * other cut is decided and computed in FP64 throughout (pivoted QR, Jacobi).  Kept spaces agree
+   * with an FP64 SVD's to 6e-14 of the largest singular value (130 cuts of the tests' networks).
+   * The gradient's forward sweep (td_grad_logprob) takes a plain FP64 Jacobi SVD of every cut. */
   /* The tensor-core Gram (bond dimensions 4..16; others use the FP64 CUDA-core Gram): each
    * value of the Gram's operands is cut into eight exact integer BF16 slices below a
    * per-column power-of-two bound (7 bits each from FP64 storage, 56 bits; 6 bits of an
@@ -98,7 +105,9 @@ typedef struct {
                               and the tensors at every segment start are checkpointed; each
                               segment but the last is swept forward again from its checkpoint
                               before its reverse sweep.  The gradient is identical either way. */
-  double svd_cutoff;       /* keep singular values s_i > svd_cutoff * s_1 */
+  double svd_cutoff;       /* keep singular values s_i > svd_cutoff * s_1 (up to 1e-11, a zip-up cut
+                              that truncates nothing else applies it to the pivots of an FP64 QR:
+                              values within a factor of a few of the cutoff may go either way) */
   double multiplet_rtol;   /* a cut inside s_k - s_{k+1} <= rtol * s_1 drops the multiplet */
   double gram_cutoff;      /* drop Gram eigen-directions below gram_cutoff * max eigenvalue;
                               negative: 1e-15 */
