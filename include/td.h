@@ -66,7 +66,8 @@ typedef enum {
    * error -- its kept space starts from an FP32 pivoted QR and Jacobi and is corrected by Newton
    * steps with FP64 residuals until the residual is at FP64 rounding (below 5e-16 of the largest
    * singular value, or below 2e-14 and no longer falling); the steps' corrections are FP32.  Every
-   * other cut is decided and computed in FP64 throughout (pivoted QR, Jacobi).  Kept spaces agree
+   * other cut is decided and computed in FP64 throughout (pivoted QR; Jacobi unless the pivots
+   * already decide that only values below svd_cutoff go).  Kept spaces agree
    * with an FP64 SVD's to 6e-14 of the largest singular value (130 cuts of the tests' networks).
    * The gradient's forward sweep (td_grad_logprob) takes a plain FP64 Jacobi SVD of every cut. */
   /* The tensor-core Gram (bond dimensions 4..16; others use the FP64 CUDA-core Gram): each
@@ -105,9 +106,7 @@ typedef struct {
                               and the tensors at every segment start are checkpointed; each
                               segment but the last is swept forward again from its checkpoint
                               before its reverse sweep.  The gradient is identical either way. */
-  double svd_cutoff;       /* keep singular values s_i > svd_cutoff * s_1 (up to 1e-11, a zip-up cut
-                              that truncates nothing else applies it to the pivots of an FP64 QR:
-                              values within a factor of a few of the cutoff may go either way) */
+  double svd_cutoff;       /* keep singular values s_i > svd_cutoff * s_1 */
   double multiplet_rtol;   /* a cut inside s_k - s_{k+1} <= rtol * s_1 drops the multiplet */
   double gram_cutoff;      /* drop Gram eigen-directions below gram_cutoff * max eigenvalue;
                               negative: 1e-15 */

@@ -25,8 +25,8 @@
 //     sigma_1; and it checks itself (the residual has to fall to FP64 rounding).
 //   * cut_rank (rank <= chi_mps: nothing to truncate): FP64 pivoted QR of M, stopped at the first
 //     pivot below svd_cutoff times the largest: U = Q, carry = R.  No SVD.  A pivot is not a singular
-//     value -- it can be off by a factor of a few --, so this path is for cutoffs that only drop what is
-//     next to rounding anyway (kCutRankCutoff).
+//     value, so it applies where the pivots leave no doubt about which values the cutoff keeps
+//     (cut_rank_decided).
 //   * cut_full (steep spectra, cuts inside a multiplet, larger cutoffs): as 1 and 2 in FP64 throughout;
 //     every singular value, so the keep rule is decided on them.
 // Measured against numpy's SVD on 130 cuts of the tests' networks: U U^T M of cut_topk differs by
@@ -938,10 +938,17 @@ static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, 
   return ok;
 }
 
-// Largest svd_cutoff that may be applied to pivots in place of singular values.  The oracle with pivots
-// (chi_mps 16 and 64, five networks) is within 2e-13 of the keep rule in log p at cutoffs up to 1e-8, 1e-5 off
-// at 1e-4 and 1e-2 off at 3e-2; the line stands well below the first and above the default, 1e-12.
-constexpr double kCutRankCutoff = 1e-11;
+// Whether a pivoted QR of n columns decides which singular values lie above cutoff times the largest: first2 and
+// last2 the squares of the first and the last kept pivot, rest2 that of the pivot it stopped at (0: none).
+// The largest value s_1 is between the first pivot and sqrt(n) times it.  The dropped ones are at most the norm
+// of what is left, sqrt(n rest2), and below the cutoff where that is.  The last kept one is rarely more than ten
+// times below its pivot (the bound is exponential, but not met in practice), so 1e3 cutoff leaves sqrt(n) and that
+// to spare.  Deciding on pivots alone moved log P of unlikely syndromes by 1e-9 at the default cutoff (2 of 1500
+// random networks) and by up to 1e-2 at cutoffs of 1e-3 and above.
+__device__ __forceinline__ bool cut_rank_decided(double first2, double last2, double rest2, int n, double cutoff) {
+  const double c2 = cutoff * cutoff * first2;
+  return last2 > 1e6 * c2 && n * rest2 <= c2;
+}
 
 // Householder QR with column pivoting of the m x n matrix X (row-major, ld n; destroyed), m <= 64 or so:
 // a thread per column, so that every FP64 instruction works on 32 columns (a column per warp leaves
@@ -1017,13 +1024,15 @@ static __device__ __noinline__ int cut_qrcp_cols(Team tm, double* X, int m, int 
 
 // Cut of rank <= most (nothing to truncate): X = M (m x n, row-major; destroyed); U (m x r) into An
 // (row-major), the carry R (r x n) into Cn; Qs: most x m scratch, vr: 4 most, nrm: n, all FP64.  Returns
-// r, or -1 when more than `most` pivots lie above the cutoff.
+// r, or -1 when more than `most` pivots lie above the cutoff or the pivots do not decide the rank.
 static __device__ __noinline__ int cut_rank(Team tm, double* X, int m, int n, int most, double cutoff, double* An, double* Cn,
                                             double* Qs, double* vr, double* nrm, CutBuf& b, double* s0) {
   double left;
   const int q = m < n ? m : n;
   const int r = cut_qrcp_cols(tm, X, m, n, cutoff * cutoff, most < q ? most : q, vr, nrm, b.taken, b.keys, left);
-  if (r == 0 || (r < q && left > cutoff * cutoff)) return -1;
+  if (r == 0) return -1;
+  const double first = vr[2], last = vr[4 * r - 2];   // R[j][j] of the first and the last step
+  if (!cut_rank_decided(first * first, last * last, r < q ? left * (first * first) : 0.0, n, cutoff)) return -1;
   const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
   for (int kk = warp; kk < r; kk += nw) {   // Q e_kk = H_0 ... H_kk e_kk, a warp per column
     double* x = Qs + (size_t)kk * m;

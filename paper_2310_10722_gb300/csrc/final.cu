@@ -177,7 +177,7 @@ static __device__ __noinline__ int cut(Team tm, const FinalArgs& fa, const doubl
       }
     }
   }
-  if (k < 0 && r32 <= cm && fa.svd_cutoff <= kCutRankCutoff) {
+  if (k < 0 && r32 <= cm) {
     const int64_t need_v = 8 * (4 * (int64_t)kk + n), need_q = 8 * (int64_t)kk * m, need_x = 8 * (int64_t)m * n;
     if (need_v + need_q <= wleft) {
       const bool xs = need_v + need_q + need_x <= pool;
