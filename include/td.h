@@ -65,10 +65,10 @@ typedef enum {
    * resolves a cut -- which values are kept under both truncation rules, with room for FP32's
    * error -- its kept space starts from an FP32 pivoted QR and Jacobi and is corrected by Newton
    * steps with FP64 residuals until the residual is at FP64 rounding (below 5e-16 of the largest
-   * singular value, or below 2e-14 and no longer falling); the steps' corrections are FP32.  Every
-   * other cut is decided and computed in FP64 throughout (pivoted QR; Jacobi unless the pivots
-   * already decide that only values below svd_cutoff go).  Kept spaces agree
-   * with an FP64 SVD's to 6e-14 of the largest singular value (130 cuts of the tests' networks).
+   * singular value, less next to a multiplet; or below 2e-14 and no longer falling); the steps'
+   * corrections are FP32.  Every other cut is decided and computed in FP64 throughout (pivoted QR;
+   * Jacobi unless the pivots already decide that only values below svd_cutoff go).  Kept spaces
+   * agree with an FP64 SVD's to 6e-14 of the largest singular value (130 cuts of the tests' networks).
    * The gradient's forward sweep (td_grad_logprob) takes a plain FP64 Jacobi SVD of every cut. */
   /* The tensor-core Gram (bond dimensions 4..16; others use the FP64 CUDA-core Gram): each
    * value of the Gram's operands is cut into eight exact integer BF16 slices below a

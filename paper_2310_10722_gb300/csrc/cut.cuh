@@ -848,6 +848,10 @@ static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, 
   }
   tm.sync();
   const double unit2 = ldexp(1.0, -2 * expo);
+  // the residual at which the space is right to FP64 rounding: an error in it is the residual over 1 - rho of the
+  // first vector left out, so next to a multiplet it has to fall further (or to its own rounding)
+  const float ratio = b.sg[b.ord[k]] / b.sg[b.ord[k - 1]];
+  const float done = 5e-16f * fminf(1.f, 8.f * (1.f - ratio * ratio));
   float prev = 0.f;
   bool ok = false, last = false;
   for (int it = 0; it < 10; ++it) {
@@ -896,7 +900,7 @@ static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, 
     tm.sync();
     const float res = __int_as_float(slots[1]);
     // converged: the residual at FP64 rounding (or no longer falling just above it)
-    if (res <= 5e-16f || (it > 0 && res <= 2e-14f && res > 0.1f * prev)) {
+    if (res <= done || (it > 0 && res <= 2e-14f && res > 0.1f * prev)) {
       ok = true;
       break;
     }
@@ -928,8 +932,8 @@ static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, 
       for (int i = 0; i < r - k; ++i) t += L[(size_t)b.ord[k + i] * ldl + c] * b.W[(size_t)i * k + j];
       V[c * k + j] += double(t);
     }
-    // the pass gained a factor res / prev; the next residual is predicted below rounding
-    last = it > 0 && res * (res / prev) * 8.f < 5e-16f;
+    // the pass gained a factor res / prev; the next residual is predicted below that
+    last = it > 0 && res * (res / prev) * 8.f < done;
     prev = res;
     tm.sync();
   }

@@ -47,9 +47,10 @@ def test_cuts_at_fp32_accuracy_would_be_seen(name, monkeypatch):
     assert np.abs(np.logaddexp(*out.T) - np.logaddexp(*ref.T)).max() > 10 * TOL
 
 
-def _apart(dem, det, chi, chi_mps, **kw):
+def _apart(dem, det, chi, chi_mps, schedule=(256, 2048), **kw):
     import paper_2310_10722_gb300 as td
     net = td.Network.from_dem(dem, chi=chi, chi_mps=chi_mps, **kw)
+    net.set_schedule(*schedule)
     d = torch.from_numpy(det).cuda()
     lp = net.coset_logprob(d)
     logP, _ = net.grad_logprob(d)
@@ -71,3 +72,12 @@ def test_values_next_to_the_cutoff(p, q, chi, rtol, shots, seed):
     seen in log P (1.4e-9 and 4e-10 where the pivots of a QR decide it)."""
     dem = rotated_phenomenological(7, 4, p, q)
     assert _apart(dem, sample_shots(dem, shots, seed=seed)[0], chi, 32, multiplet_rtol=rtol) < TOL
+
+
+@pytest.mark.gpu
+def test_cut_next_to_a_multiplet():
+    """A gap just above the multiplet rule's: the residual has to fall below its usual bound by the gap (8.9e-10
+    where it does not)."""
+    dem = rotated_phenomenological(7, 4, 0.03234, 0.00364)
+    det = sample_shots(dem, 3, seed=2278)[0]
+    assert _apart(dem, det, 16, 2, (512, 4096, False), multiplet_rtol=1e-4) < TOL
