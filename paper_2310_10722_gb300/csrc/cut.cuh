@@ -942,16 +942,19 @@ static __device__ __noinline__ bool cut_topk(Team tm, const double* A, int lda, 
   return ok;
 }
 
-// Whether a pivoted QR of n columns decides which singular values lie above cutoff times the largest: first2 and
-// last2 the squares of the first and the last kept pivot, rest2 that of the pivot it stopped at (0: none).
+// Whether a pivoted QR of n columns decides which singular values lie above cutoff times the largest: first and
+// last the first and the last kept pivot, left the square of the pivot it stopped at over the first's (0: none).
 // The largest value s_1 is between the first pivot and sqrt(n) times it.  The dropped ones are at most the norm
-// of what is left, sqrt(n rest2), and below the cutoff where that is.  The last kept one is rarely more than ten
-// times below its pivot (the bound is exponential, but not met in practice), so 1e3 cutoff leaves sqrt(n) and that
-// to spare.  Deciding on pivots alone moved log P of unlikely syndromes by 1e-9 at the default cutoff (2 of 1500
-// random networks) and by up to 1e-2 at cutoffs of 1e-3 and above.
-__device__ __forceinline__ bool cut_rank_decided(double first2, double last2, double rest2, int n, double cutoff) {
-  const double c2 = cutoff * cutoff * first2;
-  return last2 > 1e6 * c2 && n * rest2 <= c2;
+// of what is left, sqrt(n left) times the first pivot, and below the cutoff where that is.  The last kept one
+// is rarely more than ten times below its pivot (the bound is exponential, but not met in practice), so 1e3
+// cutoff leaves sqrt(n) and that to spare.  Deciding on pivots alone moved log P of unlikely syndromes by 1e-9
+// at the default cutoff (2 of 1500 random networks) and by up to 1e-2 at cutoffs of 1e-3 and above.  In FP32,
+// whose rounding is far below the margins (and whose range turns the square of a cutoff below 1e-19 into 0,
+// so that only exact zeros are dropped there): point d3, 1 shot 0.755 ms, 0.757 with the squares in FP64.
+__device__ __forceinline__ bool cut_rank_decided(double first, double last, double left, int n, double cutoff) {
+  const int e = (int)(((unsigned)__double2hiint(first) >> 20) & 0x7FFu) - 1023;
+  const float c = cut_f32(cutoff, 0);
+  return fabsf(cut_f32(last, e)) > 1e3f * c * fabsf(cut_f32(first, e)) && float(n) * cut_f32(left, 0) <= c * c;
 }
 
 // Householder QR with column pivoting of the m x n matrix X (row-major, ld n; destroyed), m <= 64 or so:
@@ -1035,8 +1038,8 @@ static __device__ __noinline__ int cut_rank(Team tm, double* X, int m, int n, in
   const int q = m < n ? m : n;
   const int r = cut_qrcp_cols(tm, X, m, n, cutoff * cutoff, most < q ? most : q, vr, nrm, b.taken, b.keys, left);
   if (r == 0) return -1;
-  const double first = vr[2], last = vr[4 * r - 2];   // R[j][j] of the first and the last step
-  if (!cut_rank_decided(first * first, last * last, r < q ? left * (first * first) : 0.0, n, cutoff)) return -1;
+  // R[j][j] of the first and the last step
+  if (!cut_rank_decided(vr[2], vr[4 * r - 2], r < q ? left : 0.0, n, cutoff)) return -1;
   const int lane = tm.tid & 31, warp = tm.tid >> 5, nw = tm.nt >> 5;
   for (int kk = warp; kk < r; kk += nw) {   // Q e_kk = H_0 ... H_kk e_kk, a warp per column
     double* x = Qs + (size_t)kk * m;
